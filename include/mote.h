@@ -92,7 +92,7 @@ mote_status_t mote_ternarize_pack(const void* W, int w_dtype, int64_t m, int64_t
  * device-wide synchronisation an allocation may imply.
  * The 256 exponent bins (2 KiB) that the exact sum of |w| needs live in a device array inside the
  * library image, so every GPU that loads the library carries those 2 KiB until the process ends.
- * The call itself asks for no device memory; it issues one memset and three kernels.  (The very
+ * The call itself asks for no device memory; it issues one memset and two kernels.  (The very
  * first use of the library on a device may make the CUDA runtime load the library's code there;
  * that happens once, is not specific to this call, and a caller that must avoid it warms up once
  * at start-up.)

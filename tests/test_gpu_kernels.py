@@ -47,6 +47,31 @@ def test_ternarize_pack_special_values(mote):
     assert a.item() == alpha and np.array_equal(packed.cpu().numpy(), O.pack_codes(codes))
 
 
+@pytest.mark.parametrize("shape,zeros,spread", [
+    ((1, 496), 0.0, 0),          # less than a warp's 512 elements
+    ((33, 1040), 0.9, 0),        # pruned weights, a ragged last item
+    ((64, 512), 0.0, 31),        # magnitudes on both edges of a thread's 32-binade window, and beyond
+    ((300, 4864), 0.5, 6),
+])
+def test_ternarize_pack_exact_sum_paths_and_thresholds(mote, shape, zeros, spread):
+    rng = np.random.default_rng(17)
+    W = (rng.standard_normal(shape) * 0.02 * np.exp2(rng.integers(-spread, spread + 1, size=shape))).astype(np.float32)
+    W[rng.random(shape) < zeros] = 0.0
+    # some weights on alpha/2 and on its neighbouring floats (found by iteration: they move alpha a little)
+    at = rng.permutation(W.size)[:6]
+    for _ in range(50):
+        alpha = O.ternarize(W)[1]
+        half = np.float32(alpha) / np.float32(2)
+        near = np.array([half, np.nextafter(half, np.float32(1)), np.nextafter(half, np.float32(0))], np.float32)
+        W.reshape(-1)[at] = np.concatenate([near, -near])
+        if O.ternarize(W)[1] == alpha:
+            break
+    codes, alpha = O.ternarize(W)
+    packed, a = mote.mote_ternarize_pack(torch.from_numpy(W).cuda())
+    assert a.item() == alpha
+    assert np.array_equal(packed.cpu().numpy(), O.pack_codes(codes))
+
+
 def test_ternarize_pack_bf16_input(mote):
     Wb = O.f32_to_bf16_rn(_randn((96, 320), 5, 0.02).astype(np.float32))
     codes, alpha = O.ternarize(O.bf16_to_f32(Wb))
