@@ -139,8 +139,8 @@ class ClockSampler:
 def stage_work(wl: synth.Workload, stage: str, stream_path: bool, experts_touched: float, shared_bits: int = 16,
                peaks: dict | None = None):
     """Algorithmic work of one launch of a stage: (amount, kind), kind 'int8' | 'bf16' | 'bytes'.
-    On the decode path the gate/up and down stages each cover the routed AND the shared expert and
-    are bound by the weight bytes they stream: 2-bit codes of the experts that received tokens plus
+    On the decode path (and in a short prefill, whose GEMMs run in pairs) the gate/up and down stages each
+    cover the routed AND the shared expert and are bound by the weight bytes they stream: 2-bit codes of the experts that received tokens plus
     the shared matrices (bf16, or RTN codes of shared_bits bits)."""
     P, T, d, f = wl.T * wl.k, wl.T, wl.d, wl.f
     sh_bytes = shared_bits / 8.0
@@ -364,10 +364,13 @@ def measure(ls: LayerSet, wl: synth.Workload, args, steps: int | None, rank: int
     # Every stage time carries the cost of the event pair around it (an event record serialises the
     # chain of programmatic dependent launches): the stages this path folds into a neighbour launch
     # nothing, so what they show is that cost alone.  It is taken off the stages that do launch.
-    folded = ("dispatch", "quant_x", "shared_gateup", "shared_down", "combine") if stream_path else ("combine",)
     n_l0 = len(layers)
+    # a short prefill runs the routed and the shared GEMM of a step as one launch: the shared stages launch nothing
+    paired = not stream_path and max(stage_raw["shared_gateup"], stage_raw["shared_down"]) / n_l0 < 4e-3
+    folded = (("dispatch", "quant_x", "shared_gateup", "shared_down", "combine") if stream_path
+              else ("shared_gateup", "shared_down") if paired else ("combine",))
     event_ms = min(stage_raw[k_] for k_ in folded) / n_l0
-    if event_ms * 1e3 > 4.0:                             # a "folded" stage that did launch (K-split shared down: combine): no estimate
+    if event_ms * 1e3 > 4.0:                             # a "folded" stage that did launch: no estimate
         event_ms = 0.0
     stage_ms = {k_: (0.0 if k_ in folded and v / n_l0 - event_ms < 1.5e-3 else max(v - event_ms * n_l0, 0.0))
                 for k_, v in stage_raw.items()}
@@ -393,7 +396,7 @@ def measure(ls: LayerSet, wl: synth.Workload, args, steps: int | None, rank: int
     sustained = total_ms >= SUSTAINED_MIN_MS
     n_l = len(layers)
     dom = max(stage_ms, key=stage_ms.get)
-    work, kind = stage_work(wl, dom, stream_path, experts_touched, args.shared_bits, peaks)
+    work, kind = stage_work(wl, dom, stream_path or paired, experts_touched, args.shared_bits, peaks)
     dur_s = stage_ms[dom] * 1e-3 / n_l                  # average duration of one launch of that kernel
     from paper_2506_14435_b200 import traffic
     label = workload_label(wl)
@@ -440,7 +443,7 @@ def measure(ls: LayerSet, wl: synth.Workload, args, steps: int | None, rank: int
                              "frac_of_nominal": rec["weights_touched_gbs"] / NOMINAL["hbm_gbs"],
                              "note": "all weight bytes touched (2-bit codes of the experts that received tokens + the "
                                      "shared expert) over the whole step; the stream kernels cover both"}
-    else:
+    elif not paired:
         t_routed = (stage_ms["gateup_ternary"] + stage_ms["down_ternary"]) * 1e-3 / n_l
         t_with_q = t_routed + stage_ms["quant_h"] * 1e-3 / n_l
         ops = 6.0 * wl.d * wl.f * P

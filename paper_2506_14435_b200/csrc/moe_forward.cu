@@ -378,6 +378,30 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   st = launch_quant_act(qa, true, stream);
   if (st) return st;
   stage_mark(3, stream);
+  // prefill with an RTN-coded shared expert and room in the workspace: expand the codes to bf16 once
+  SharedMat xg = sh_gate, xu = sh_up, xd = sh_down;
+  int x_bits = sh_bits;
+  auto expand_shared = [&]() -> mote_status_t {
+    if (!(sh_rtn && tensor && T >= kExpandMinTokens && ws_bytes >= pl.total_expanded)) return MOTE_OK;
+    char* e0 = base + pl.sh_codes_bf16;
+    const size_t mat = size_t(d) * f * 2;
+    ExpandArgs ea{};
+    for (int i = 0; i < 3; ++i) {
+      ea.codes[i] = static_cast<const uint4*>(i == 0 ? sh_gate.w : i == 1 ? sh_up.w : sh_down.w);
+      ea.out[i] = reinterpret_cast<uint4*>(e0 + i * mat);
+    }
+    xg.w = e0; xu.w = e0 + mat; xd.w = e0 + 2 * mat;
+    x_bits = MOTE_SHARED_BF16;                     // bf16 operands; the row scales still apply
+    return launch_expand_codes(ea, int64_t(d) * f, sh_bits, stream);
+  };
+  // Few row tiles (the shared down projection is cut along K): neither the routed nor the shared GEMM of a step fills the
+  // SMs and both are short, so they are one launch, which also saves two.  A 64-token call of a 256 x 512 layer took
+  // 43.0 us in nine launches and takes 33.0 in seven; 1536 x 8960, 8 experts: 117 -> 107 (64 tokens), 162 -> 157 (512),
+  // 228 -> 228 (1024).  With more row tiles every GEMM fills the SMs by itself, and the shared down projection's
+  // epilogue does the combine, for which the routed one has to be complete.
+  const int k_splits = tensor ? shared_down_k_splits(T, d, f) : 1;
+  const bool pair = tensor && k_splits > 1;
+  if (pair && (st = expand_shared())) return st;
   // S4 gate/up
   TernaryGemmArgs g1{};
   g1.qa = qx; g1.beta = beta_x; g1.offsets = offsets; g1.w0 = L->gate_packed; g1.w1 = L->up_packed;
@@ -385,9 +409,11 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   g1.h_bf16 = h; g1.acc0_tap = taps ? taps->acc_gate : nullptr; g1.acc1_tap = taps ? taps->acc_up : nullptr;
   if (tensor && !blockwise)   // beta_h (atomicMax target) and rowsum_h (atomicAdd target) are adjacent
     MOTE_CUDA_OK(cudaMemsetAsync(beta_h, 0, (pl.rowsum_h - pl.beta_h) + size_t(P) * 4, stream));
-  st = tensor ? launch_ternary_umma(g1, true, tiles_routed, max_mtiles_routed, rowsum_x,
-                                    reinterpret_cast<uint32_t*>(beta_h), status, stream, pdl)
-              : launch_ternary_gateup_simt(g1, stream);
+  st = pair     ? launch_umma_pair(g1, true, tiles_routed, max_mtiles_routed, rowsum_x, reinterpret_cast<uint32_t*>(beta_h), x,
+                                   xg, xu, x_bits, T, hs, tiles_shared, max_mtiles_shared, status, stream, pdl, 1)
+       : tensor ? launch_ternary_umma(g1, true, tiles_routed, max_mtiles_routed, rowsum_x,
+                                      reinterpret_cast<uint32_t*>(beta_h), status, stream, pdl)
+                : launch_ternary_gateup_simt(g1, stream);
   if (st) return st;
   stage_mark(4, stream);
   // S5 Q_a(h)
@@ -402,38 +428,23 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   TernaryGemmArgs g2{};
   g2.qa = qh; g2.beta = beta_h; g2.offsets = offsets; g2.w0 = L->down_packed; g2.alpha0 = L->alpha_down;
   g2.E = E; g2.N = d; g2.K = f; g2.P = P; g2.y = y; g2.acc0_tap = taps ? taps->acc_down : nullptr;
-  st = tensor ? launch_ternary_umma(g2, false, tiles_routed, max_mtiles_routed, rowsum_h, nullptr, status, stream, pdl)
-              : launch_ternary_down_simt(g2, stream);
+  st = pair     ? launch_umma_pair(g2, false, tiles_routed, max_mtiles_routed, rowsum_h, nullptr, hs, xd,
+                                   SharedMat{nullptr, nullptr}, x_bits, T, s, tiles_shared, max_mtiles_shared, status, stream,
+                                   pdl, k_splits)
+       : tensor ? launch_ternary_umma(g2, false, tiles_routed, max_mtiles_routed, rowsum_h, nullptr, status, stream, pdl)
+                : launch_ternary_down_simt(g2, stream);
   if (st) return st;
   stage_mark(6, stream);
   // S7 shared expert
-  // prefill with an RTN-coded shared expert and room in the workspace: expand the codes to bf16 once
-  SharedMat xg = sh_gate, xu = sh_up, xd = sh_down;
-  int x_bits = sh_bits;
-  if (sh_rtn && tensor && T >= kExpandMinTokens && ws_bytes >= pl.total_expanded) {
-    char* e0 = base + pl.sh_codes_bf16;
-    const size_t mat = size_t(d) * f * 2;
-    ExpandArgs ea{};
-    for (int i = 0; i < 3; ++i) {
-      ea.codes[i] = static_cast<const uint4*>(i == 0 ? sh_gate.w : i == 1 ? sh_up.w : sh_down.w);
-      ea.out[i] = reinterpret_cast<uint4*>(e0 + i * mat);
-    }
-    st = launch_expand_codes(ea, int64_t(d) * f, sh_bits, stream);
-    if (st) return st;
-    xg.w = e0; xu.w = e0 + mat; xd.w = e0 + 2 * mat;
-    x_bits = MOTE_SHARED_BF16;                     // bf16 operands; the row scales still apply
-  }
-  st = tensor ? launch_shared_umma(x, xg, xu, x_bits, true, T, d, f, hs, tiles_shared, max_mtiles_shared,
-                                   status, nullptr, stream, pdl)
-              : launch_shared_gateup_simt(x, sh_gate, sh_up, sh_bits, T, d, f, hs, stream);
+  if (!pair && (st = expand_shared())) return st;
+  st = pair     ? MOTE_OK
+       : tensor ? launch_shared_umma(x, xg, xu, x_bits, true, T, d, f, hs, tiles_shared, max_mtiles_shared,
+                                     status, nullptr, stream, pdl)
+                : launch_shared_gateup_simt(x, sh_gate, sh_up, sh_bits, T, d, f, hs, stream);
   if (st) return st;
   stage_mark(7, stream);
-  const int k_splits = tensor ? shared_down_k_splits(T, d, f) : 1;
-  if (tensor && k_splits > 1) {
-    // few row tiles: the shared down projection is cut along K, its partial outputs are added by the combine
-    st = launch_shared_umma(hs, xd, SharedMat{nullptr, nullptr}, x_bits, false, T, f, d, s, tiles_shared,
-                            max_mtiles_shared, status, nullptr, stream, pdl, k_splits);
-    if (st) return st;
+  if (pair) {
+    // the shared down projection was cut along K; its partial outputs are added by the combine
     stage_mark(8, stream);
     st = launch_combine(s, y, topk_w, perm, residual, T, d, k, out, stream, pdl, k_splits);
     if (st) return st;

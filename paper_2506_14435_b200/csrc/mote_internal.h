@@ -103,6 +103,12 @@ mote_status_t launch_shared_umma(const void* act, const SharedMat& w0, const Sha
                                  int64_t T, int K, int N, void* out, const int4* tiles, int max_mtiles,
                                  uint32_t* status, const CombineArgs* comb, cudaStream_t stream, bool pdl = false,
                                  int k_splits = 1);
+// The routed GEMM and the shared expert's GEMM of the same step (gate/up, or down) as one launch; `act`, w0, w1, bits, T,
+// out, tiles_shared, k_splits: the shared one's, as in launch_shared_umma.
+mote_status_t launch_umma_pair(const TernaryGemmArgs& g, bool gateup, const int4* tiles_routed, int max_mtiles_routed,
+                               const int32_t* rowsum, uint32_t* beta_out_bits, const void* act, const SharedMat& w0,
+                               const SharedMat& w1, int bits, int64_t T, void* out, const int4* tiles_shared,
+                               int max_mtiles_shared, uint32_t* status, cudaStream_t stream, bool pdl, int k_splits);
 // Diagnostic: one CTA waits on an mbarrier that nothing arrives at, with the GEMM kernels' bounded
 // wait and teardown; after limit_ns it raises *status and returns.
 mote_status_t launch_bounded_wait_selftest(uint32_t* status, uint64_t limit_ns, cudaStream_t stream);

@@ -109,6 +109,20 @@ struct ModeTraits {
                                   (kUnpack ? size_t(kStagesP) * kStageP : 0) + kEpiStage + sizeof(PipeBarriers);
 };
 
+// What a CTA of one GEMM (SMODE < 0) or of a pair of GEMMs lays out in shared memory.
+template <int MODE, int SMODE>
+struct PairTraits {
+  using TR = ModeTraits<MODE>; using TS = ModeTraits<SMODE>;
+  static constexpr bool kGateUp = TR::kGateUp, kUnpack = true;
+  static constexpr int kStages = kStagesTernary;
+  static constexpr int kStageP = std::max(TR::kStageP, TS::kUnpack ? TS::kStageP : 0);
+  static constexpr int kStagesP = TS::kRtnBits == 8 ? 3 : 4;
+  static constexpr size_t kEpiStage = TS::kEpiStage;
+  static constexpr size_t kSmem = 1024 + size_t(kStages) * (kStageA + kStageB) + size_t(kStagesP) * kStageP + kEpiStage + sizeof(PipeBarriers);
+};
+template <int MODE>
+struct PairTraits<MODE, -1> : ModeTraits<MODE> {};
+
 // Item order.  The CTAs of the grid work on neighbouring items at the same time, and the operand
 // those items share is the one L2 serves to all of them from a single HBM read.
 //   gate/up: row tile fastest -- concurrent items share the (small) weight tile; the token operand
@@ -181,12 +195,445 @@ static __device__ __noinline__ float glu_h_rare(int acc_g, int acc_u, float c_g,
 }
 
 // ------------------------------------------------------------------------------------------------
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
-umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
-                 const __grid_constant__ CUtensorMap tm_b1, const UmmaArgs a) {
+// What the warps of a CTA do for one item, by role.  A ring of `n` stages is walked with the parity of its barriers'
+// phase; false: a bounded wait ran out.
+// ------------------------------------------------------------------------------------------------
+struct RingPos {
+  uint32_t stage = 0, phase = 0;
+  __device__ __forceinline__ void next(uint32_t n) {
+    if (++stage == n) { stage = 0; phase ^= 1; }
+  }
+};
+
+// the token operand, and the weights where they are bf16
+template <int MODE, int S>
+__device__ __forceinline__ bool load_operands(const CUtensorMap& tm_a, const CUtensorMap& tm_b0, const CUtensorMap& tm_b1,
+                                              const UmmaArgs& a, int item, int n_mtiles, int n_whole, uint32_t sA, uint32_t sB,
+                                              PipeBarriers* bars, RingPos& p) {
   using TR = ModeTraits<MODE>;
-  constexpr int S = TR::kStages;
+  volatile int* abort_flag = &bars->abort_flag;
+  int4 tile; int n_tile, half;
+  decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
+  const int width = half < 0 ? a.bn : 128;
+  const int b_row = (a.b_rows_per_expert ? tile.x * a.b_rows_per_expert : 0) +
+                    n_tile * (TR::kGateUp ? a.bn / 2 : a.bn) + (half > 0 ? 128 : 0);
+  int kb, ke;
+  item_k_range<TR::kGateUp>(a, item, kb, ke);
+  for (int ks = kb; ks < ke; ++ks) {
+    if (!mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, abort_flag)) return false;
+    const uint32_t bar = smem_u32(&bars->full_a[p.stage]);
+    if (TR::kTernary) {
+      mbar_expect_tx(bar, kStageA);
+      tma_load_2d(sA + p.stage * kStageA, &tm_a, ks * 128, tile.y, bar);
+    } else if (TR::kRtn) {
+      mbar_expect_tx(bar, kStageA);
+      tma_load_2d(sA + p.stage * kStageA, &tm_a, ks * 64, tile.y, bar);
+    } else {
+      mbar_expect_tx(bar, kStageA + width * 128);
+      tma_load_2d(sA + p.stage * kStageA, &tm_a, ks * 64, tile.y, bar);
+      if (TR::kGateUp) {
+        tma_load_2d(sB + p.stage * kStageB, &tm_b0, ks * 64, b_row, bar);
+        tma_load_2d(sB + p.stage * kStageB + 128 * 128, &tm_b1, ks * 64, b_row, bar);
+      } else {
+        tma_load_2d(sB + p.stage * kStageB, &tm_b0, ks * 64, b_row, bar);
+        if (width > 128) tma_load_2d(sB + p.stage * kStageB + 128 * 128, &tm_b1, ks * 64, b_row + 128, bar);
+      }
+    }
+    p.next(S);
+  }
+  return true;
+}
+
+// weight codes
+template <int MODE, int kStagesP, int kStageP>
+__device__ __forceinline__ bool load_codes(const CUtensorMap& tm_b0, const CUtensorMap& tm_b1, const UmmaArgs& a, int item, int n_mtiles, int n_whole,
+                                           uint32_t sP, PipeBarriers* bars, RingPos& p) {
+  using TR = ModeTraits<MODE>;
+  volatile int* abort_flag = &bars->abort_flag;
+  constexpr int kRB = TR::kCodeRowBytes;
+  int4 tile; int n_tile, half;
+  decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
+  const int width = half < 0 ? a.bn : 128;
+  const int b_row = tile.x * a.b_rows_per_expert + n_tile * (TR::kGateUp ? a.bn / 2 : a.bn) + (half > 0 ? 128 : 0);
+  int kb, ke;
+  item_k_range<TR::kGateUp>(a, item, kb, ke);
+  for (int ks = kb; ks < ke; ++ks) {
+    if (!mbar_wait(smem_u32(&bars->empty_p[p.stage]), p.phase ^ 1, abort_flag)) return false;
+    const uint32_t bar = smem_u32(&bars->full_p[p.stage]);
+    mbar_expect_tx(bar, width * kRB);
+    const uint32_t dst = sP + p.stage * kStageP;
+    if (TR::kGateUp) {
+      tma_load_2d(dst, &tm_b0, ks * kRB, b_row, bar);
+      tma_load_2d(dst + 128 * kRB, &tm_b1, ks * kRB, b_row, bar);
+    } else {
+      tma_load_2d(dst, &tm_b0, ks * kRB, b_row, bar);
+      if (width > 128) tma_load_2d(dst + 128 * kRB, &tm_b1, ks * kRB, b_row + 128, bar);
+    }
+    p.next(kStagesP);
+  }
+  return true;
+}
+
+// kWaitU: the unpackers announce every pipeline stage
+template <int MODE, int S, bool kWaitU>
+__device__ __forceinline__ bool issue_mmas(const UmmaArgs& a, int item, int n_whole, int local, uint32_t tmem_base, uint32_t sA,
+                                           uint32_t sB, PipeBarriers* bars, RingPos& p) {
+  using TR = ModeTraits<MODE>;
+  volatile int* abort_flag = &bars->abort_flag;
+  const uint32_t idesc_whole = TR::kTernary ? make_idesc(2, 1, 0, kBM, (uint32_t)a.bn)     // s32 += s8 * u8
+                                            : make_idesc(1, 1, 1, kBM, (uint32_t)a.bn);    // f32 += bf16 * bf16
+  const uint32_t idesc_half = TR::kTernary ? make_idesc(2, 1, 0, kBM, 128u) : make_idesc(1, 1, 1, kBM, 128u);
+  const int buf = local & 1;
+  const uint32_t use = (uint32_t)(local >> 1);
+  if (!mbar_wait(smem_u32(&bars->tmem_empty[buf]), (use & 1) ^ 1, abort_flag)) return false;
+  tc_fence_after();
+  const uint32_t d_tmem = tmem_base + buf * 256;
+  const uint32_t idesc = (!TR::kGateUp && item >= n_whole) ? idesc_half : idesc_whole;
+  int kb, ke;
+  item_k_range<TR::kGateUp>(a, item, kb, ke);
+  for (int ks = kb; ks < ke; ++ks) {
+    if (!mbar_wait(smem_u32(&bars->full_a[p.stage]), p.phase, abort_flag)) return false;
+    if (kWaitU)
+      if (!mbar_wait(smem_u32(&bars->full_u[p.stage]), p.phase, abort_flag)) return false;
+    tc_fence_after();
+    const uint64_t da = smem_desc_sw128(sA + p.stage * kStageA);
+    const uint64_t db = smem_desc_sw128(sB + p.stage * kStageB);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t acc = (ks > kb || j > 0) ? 1u : 0u;
+      if (TR::kTernary) mma_i8(d_tmem, da + 2 * j, db + 2 * j, idesc, acc);
+      else mma_f16(d_tmem, da + 2 * j, db + 2 * j, idesc, acc);
+    }
+    mma_commit(smem_u32(&bars->empty[p.stage]));
+    p.next(S);
+  }
+  mma_commit(smem_u32(&bars->tmem_full[buf]));
+  return true;
+}
+
+// 2-bit -> int8 for the ternary experts; int8 / 4-bit -> bf16 for an RTN-coded shared expert.  group 0 (warps 4-7)
+// expands the even pipeline steps, group 1 (warps 8-11) the odd ones.  p, q: positions in the rings of stages and codes
+template <int MODE, int S, int kStagesP, int kStageP>
+__device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_whole, int group, uint8_t* genB,
+                                             const uint8_t* genP, PipeBarriers* bars, RingPos& p, RingPos& q, uint32_t& step) {
+  using TR = ModeTraits<MODE>;
+  volatile int* abort_flag = &bars->abort_flag;
+  const int tid = (threadIdx.x - 128) & 127, lane = threadIdx.x & 31;
+  if constexpr (!TR::kUnpack) {                    // bf16 weights among items with codes: only the announcements
+    int kb, ke;
+    item_k_range<TR::kGateUp>(a, item, kb, ke);
+    for (int ks = kb; ks < ke; ++ks, ++step, p.next(S)) {
+      if ((step & 1u) != (uint32_t)group) continue;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, abort_flag))) return false;
+      if (lane == 0) mbar_arrive(smem_u32(&bars->full_u[p.stage]));
+    }
+    return true;
+  }
+  // chunks of 16 code bytes, spread over 128 threads
+  const int n_chunks = ((!TR::kGateUp && item >= n_whole) ? 128 : a.bn) * (TR::kCodeRowBytes / 16);
+  int kb, ke;
+  item_k_range<TR::kGateUp>(a, item, kb, ke);
+  for (int ks = kb; ks < ke; ++ks, ++step) {
+    if ((step & 1u) == (uint32_t)group) {
+      const bool ok = mbar_wait(smem_u32(&bars->full_p[q.stage]), q.phase, abort_flag) &&
+                      mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, abort_flag);
+      if (!__all_sync(0xffffffffu, ok)) return false;
+      const uint8_t* src = genP + q.stage * kStageP;
+      uint8_t* dst = genB + p.stage * kStageB;
+      // batches of four chunks per thread, all loads of a batch ahead of its conversions
+      for (int c0 = tid; c0 < n_chunks; c0 += 128 * 4) {
+        uint4 wv[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const int c = c0 + b * 128;
+          if (c < n_chunks) wv[b] = *reinterpret_cast<const uint4*>(src + c * 16);
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const int c = c0 + b * 128;
+          if (c >= n_chunks) break;
+          const uint32_t pw[4] = {wv[b].x, wv[b].y, wv[b].z, wv[b].w};
+          if (TR::kRtnBits == 8) {
+            // 16 int8 codes -> two 16-byte pieces of 8 bf16 each
+            const int r = c >> 2, quarter = c & 3;
+            uint8_t* row = dst + (r >> 3) * 1024 + (r & 7) * 128;
+            uint32_t e[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s8x4_to_bf16x2(pw[j], e[2 * j], e[2 * j + 1]);
+            *reinterpret_cast<uint4*>(row + (((quarter * 2) ^ (r & 7)) << 4)) = make_uint4(e[0], e[1], e[2], e[3]);
+            *reinterpret_cast<uint4*>(row + (((quarter * 2 + 1) ^ (r & 7)) << 4)) = make_uint4(e[4], e[5], e[6], e[7]);
+          } else {
+            const int r = c >> 1, half = c & 1;
+            uint8_t* row = dst + (r >> 3) * 1024 + (r & 7) * 128;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              uint4 o;
+              if (TR::kRtnBits == 4) {
+                // 8 four-bit codes -> one 16-byte piece of 8 bf16
+                uint32_t e[4];
+                u4x8_to_bf16x2(pw[j], e);
+                o = make_uint4(e[0], e[1], e[2], e[3]);
+              } else {
+                o.x = pw[j] & 0x03030303u;
+                o.y = (pw[j] >> 2) & 0x03030303u;
+                o.z = (pw[j] >> 4) & 0x03030303u;
+                o.w = (pw[j] >> 6) & 0x03030303u;
+              }
+              *reinterpret_cast<uint4*>(row + (((half * 4 + j) ^ (r & 7)) << 4)) = o;
+            }
+          }
+        }
+      }
+      fence_proxy_async_smem();                // generic-proxy writes -> visible to the MMA
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(smem_u32(&bars->full_u[p.stage]));
+        mbar_arrive(smem_u32(&bars->empty_p[q.stage]));
+      }
+    }
+    p.next(S);
+    q.next(kStagesP);
+  }
+  return true;
+}
+
+template <int MODE>
+__device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mtiles, int n_whole, int local, uint32_t tmem_base,
+                                          uint8_t* genE, PipeBarriers* bars) {
+  using TR = ModeTraits<MODE>;
+  volatile int* abort_flag = &bars->abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q = warp & 3;                          // TMEM lane quarter this warp may read
+  const int chalf = (warp - 12) >> 2;              // which half of the tile's columns
+  const int r_in_tile = q * 32 + lane;
+  int4 tile; int n_tile, half;
+  decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
+  int kb_, ke_;
+  const int split = item_k_range<TR::kGateUp>(a, item, kb_, ke_);
+  const int buf = local & 1;
+  const uint32_t use = (uint32_t)(local >> 1);
+  const bool ok = mbar_wait(smem_u32(&bars->tmem_full[buf]), use & 1, abort_flag);
+  if (!__all_sync(0xffffffffu, ok)) return false;
+  tc_fence_after();
+  const bool row_ok = r_in_tile < tile.z;
+  const int64_t row = int64_t(tile.y) + r_in_tile;
+  const uint32_t t_row = tmem_base + (uint32_t(q * 32) << 16) + buf * 256;
+  float c0 = 0.f, c1 = 0.f;
+  int rs = 0;
+  if (TR::kTernary && row_ok) {
+    const float beta = fmaxf(a.beta[row], kEpsScale);
+    rs = a.rowsum[row];
+    c0 = dequant_scale(a.alpha0[tile.x], beta);
+    if (TR::kGateUp) c1 = dequant_scale(a.alpha1[tile.x], beta);
+  }
+  if (TR::kGateUp) {
+    const int col0 = n_tile * 128;
+    const bool row_fast = __fmul_rn(c0, c1) > 1e-12f;
+    const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;
+    float hmax = 0.0f;                           // max |h| (before the bf16 rounding, which is monotonic)
+    constexpr int kCols = TR::kEpiCols, kPitch = TR::kEpiPitch;
+    constexpr int kLanesPerRow = kCols * 2 / 16, kRowsPerStore = 32 / kLanesPerRow;
+    uint8_t* stg = genE + (warp - 12) * 32 * kPitch;
+#pragma unroll 1
+    for (int cr = chalf * 64; cr < chalf * 64 + 64; cr += kCols) {
+#pragma unroll 1
+      for (int c = cr; c < cr + kCols; c += 16) {
+        uint32_t rg[16], ru[16];
+        tmem_ld_32x32b_x16(t_row + c, rg);
+        tmem_ld_32x32b_x16(t_row + 128 + c, ru);
+        tmem_wait_ld();
+        if (row_ok) {
+          float hv[16];
+          if (TR::kTernary) {
+            uint32_t redo_mask = 0u;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              bool redo;
+              hv[j] = glu_h_fast_biased(rg[j], ru[j], acc_bias, c0, c1, redo);
+              if (redo) redo_mask |= 1u << j;
+            }
+            if (!row_fast) redo_mask = 0xFFFFu;
+            if (redo_mask) {                     // mostly one element: look at four at a time
+#pragma unroll
+              for (int j0 = 0; j0 < 16; j0 += 4)
+                if ((redo_mask >> j0) & 0xFu) {
+#pragma unroll
+                  for (int j = j0; j < j0 + 4; ++j)
+                    if ((redo_mask >> j) & 1u) hv[j] = glu_h_rare((int)rg[j] - rs, (int)ru[j] - rs, c0, c1);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) hmax = fmaxf(hmax, fabsf(hv[j]));
+          } else if (TR::kRtn || a.alpha0 != nullptr) {
+            // RTN-coded shared expert (codes expanded here, or beforehand): row scales of the
+            // gate and up matrices = scales of this tile's output columns
+            const float4* sgp = reinterpret_cast<const float4*>(a.alpha0 + col0 + c);
+            const float4* sup = reinterpret_cast<const float4*>(a.alpha1 + col0 + c);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              const float4 sg = __ldg(sgp + v), su = __ldg(sup + v);
+              const float sgv[4] = {sg.x, sg.y, sg.z, sg.w}, suv[4] = {su.x, su.y, su.z, su.w};
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const float g = __uint_as_float(rg[4 * v + u]) * sgv[u];
+                hv[4 * v + u] = __uint_as_float(ru[4 * v + u]) * suv[u] * silu_fast(g);
+              }
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float g = __uint_as_float(rg[j]);
+              hv[j] = __uint_as_float(ru[j]) * silu_fast(g);
+            }
+          }
+          uint32_t packed[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) packed[j] = pack_bf16x2(hv[2 * j], hv[2 * j + 1]);
+          if (TR::kTernary) {
+            // the thread's 16 bf16 values are one 32-byte sector of its row: one store
+            st_global_v8(reinterpret_cast<uint16_t*>(a.out) + row * a.n_out + col0 + c, packed[0], packed[1], packed[2],
+                         packed[3], packed[4], packed[5], packed[6], packed[7]);
+          } else {
+            uint4* sdst = reinterpret_cast<uint4*>(stg + lane * kPitch + (c - cr) * 2);
+            sdst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+            sdst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+          }
+          if (TR::kTernary && a.tap0) {
+            int4* t0 = reinterpret_cast<int4*>(a.tap0 + row * a.n_out + col0 + c);
+            int4* t1 = reinterpret_cast<int4*>(a.tap1 + row * a.n_out + col0 + c);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              t0[v] = make_int4((int)rg[4 * v] - rs, (int)rg[4 * v + 1] - rs, (int)rg[4 * v + 2] - rs, (int)rg[4 * v + 3] - rs);
+              t1[v] = make_int4((int)ru[4 * v] - rs, (int)ru[4 * v + 1] - rs, (int)ru[4 * v + 2] - rs, (int)ru[4 * v + 3] - rs);
+            }
+          }
+        }
+      }
+      if (!TR::kTernary) {
+        __syncwarp();
+        // the warp's 32 rows x kCols columns leave as whole row segments (kCols * 2 bytes each)
+#pragma unroll
+        for (int r0 = 0; r0 < 32; r0 += kRowsPerStore) {
+          const int r = r0 + lane / kLanesPerRow, piece = lane % kLanesPerRow;
+          if (q * 32 + r < tile.z) {
+            const uint4 v = *reinterpret_cast<const uint4*>(stg + r * kPitch + piece * 16);
+            uint16_t* orow = reinterpret_cast<uint16_t*>(a.out) + (int64_t(tile.y) + q * 32 + r) * a.n_out + col0 + cr;
+            reinterpret_cast<uint4*>(orow)[piece] = v;
+          }
+        }
+        __syncwarp();
+      }
+    }
+    // bits of non-negative floats order like unsigned integers; bf16_rn(max) = max(bf16_rn)
+    if (TR::kTernary && row_ok && a.beta_out_bits) {
+      const uint32_t hb = f32_to_bf16_bits(hmax) << 16;
+      if (hb) atomicMax(a.beta_out_bits + row, hb);
+    }
+  } else {
+    const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;   // see glu_h_fast_biased
+    const int width = half < 0 ? a.bn : 128;
+    const int col0 = n_tile * a.bn + (half > 0 ? 128 : 0);
+    const int cbeg = chalf * (width / 2), cend = cbeg + width / 2;
+    const bool combine = !TR::kTernary && a.comb_out != nullptr;
+    float cw[MOTE_MAX_TOPK];
+    const float* cy[MOTE_MAX_TOPK];
+    if (combine && row_ok) {
+#pragma unroll
+      for (int j = 0; j < MOTE_MAX_TOPK; ++j)
+        if (j < a.comb_k) {
+          cw[j] = a.comb_w[row * a.comb_k + j];
+          cy[j] = a.comb_y + int64_t(a.comb_perm[row * a.comb_k + j]) * a.n_out + col0;
+        }
+    }
+#pragma unroll 1
+    for (int c = cbeg; c < cend; c += 16) {
+      uint32_t ra[16];
+      tmem_ld_32x32b_x16(t_row + c, ra);
+      tmem_wait_ld();
+      if (row_ok) {
+        float o[16];
+#pragma unroll
+        for (int v = 0; v < 16; ++v)
+          o[v] = TR::kTernary ? __fmul_rn(__fsub_rn(__uint_as_float(ra[v] + acc_bias), kMagic), c0)   // fl32(acc - rs) * c0
+                              : __uint_as_float(ra[v]);
+        if (TR::kRtn || (!TR::kTernary && a.alpha0 != nullptr)) {
+          const float4* sp = reinterpret_cast<const float4*>(a.alpha0 + col0 + c);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const float4 sc = __ldg(sp + v);
+            o[4 * v] *= sc.x; o[4 * v + 1] *= sc.y; o[4 * v + 2] *= sc.z; o[4 * v + 3] *= sc.w;
+          }
+        }
+        if (a.out) {
+          float* dst = reinterpret_cast<float*>(a.out) + split * a.split_stride + row * a.n_out + col0 + c;
+#pragma unroll
+          for (int v = 0; v < 2; ++v)
+            st_global_v8(dst + 8 * v, __float_as_uint(o[8 * v]), __float_as_uint(o[8 * v + 1]), __float_as_uint(o[8 * v + 2]),
+                         __float_as_uint(o[8 * v + 3]), __float_as_uint(o[8 * v + 4]), __float_as_uint(o[8 * v + 5]),
+                         __float_as_uint(o[8 * v + 6]), __float_as_uint(o[8 * v + 7]));
+        }
+        if (TR::kTernary && a.tap0) {
+          int4* t0 = reinterpret_cast<int4*>(a.tap0 + row * a.n_out + col0 + c);
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            t0[v] = make_int4((int)ra[4 * v] - rs, (int)ra[4 * v + 1] - rs, (int)ra[4 * v + 2] - rs, (int)ra[4 * v + 3] - rs);
+        }
+        if (combine) {
+          // fp32, slots in ascending j, then the residual, one bf16 rounding
+#pragma unroll
+          for (int j = 0; j < MOTE_MAX_TOPK; ++j)
+            if (j < a.comb_k) {
+#pragma unroll
+              for (int v = 0; v < 2; ++v) {
+                uint32_t yv[8];
+                ld_global_v8(cy[j] + c + 8 * v, yv);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) o[8 * v + u] = fmaf(cw[j], __uint_as_float(yv[u]), o[8 * v + u]);
+              }
+            }
+          if (a.comb_res) {
+            uint32_t rw[8];
+            if (a.comb_wide) {
+              ld_global_v8(a.comb_res + row * a.n_out + col0 + c, rw);
+            } else {
+              const uint4* rp = reinterpret_cast<const uint4*>(a.comb_res + row * a.n_out + col0 + c);
+              const uint4 r0 = rp[0], r1 = rp[1];
+              rw[0] = r0.x; rw[1] = r0.y; rw[2] = r0.z; rw[3] = r0.w; rw[4] = r1.x; rw[5] = r1.y; rw[6] = r1.z; rw[7] = r1.w;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) { o[2 * u] += bf16_lo(rw[u]); o[2 * u + 1] += bf16_hi(rw[u]); }
+          }
+          uint32_t pk[8];
+#pragma unroll
+          for (int v = 0; v < 8; ++v) pk[v] = f32_to_bf16_bits(o[2 * v]) | (f32_to_bf16_bits(o[2 * v + 1]) << 16);
+          if (a.comb_wide) {
+            st_global_v8(a.comb_out + row * a.n_out + col0 + c, pk[0], pk[1], pk[2], pk[3], pk[4], pk[5], pk[6], pk[7]);
+          } else {
+            uint4* od = reinterpret_cast<uint4*>(a.comb_out + row * a.n_out + col0 + c);
+            od[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            od[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+          }
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(smem_u32(&bars->tmem_empty[buf]));
+  return true;
+}
+
+// ------------------------------------------------------------------------------------------------
+// The CTA's walk over its items: all of mode MODE, or (pair of GEMMs) routed items of mode MODE and shared items of
+// mode SMODE.  A pair takes the longer items first: gate/up the shared ones (bf16 rows are eight times as long as 2-bit
+// ones), down the routed ones (the shared ones are cut along K).
+template <int MODE, int SMODE>
+__device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensorMap& tm_b0, const CUtensorMap& tm_b1, const UmmaArgs& a,
+                                         const CUtensorMap& ts_a, const CUtensorMap& ts_b0, const CUtensorMap& ts_b1, const UmmaArgs& as) {
+  using TR = PairTraits<MODE, SMODE>;
+  constexpr bool kPair = SMODE >= 0;
+  constexpr int kS = kPair ? SMODE : MODE;
+  constexpr int S = TR::kStages, kStagesP = TR::kStagesP, kStageP = TR::kStageP;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -195,7 +642,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   const uint32_t sP = sB + S * kStageB;
   uint8_t* genB = smem_gen + S * kStageA;
   uint8_t* genP = genB + S * kStageB;
-  uint8_t* genE = genP + (TR::kUnpack ? TR::kStagesP * TR::kStageP : 0);
+  uint8_t* genE = genP + (TR::kUnpack ? kStagesP * kStageP : 0);
   PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(genE + TR::kEpiStage);
   volatile int* abort_flag = &bars->abort_flag;
 
@@ -218,6 +665,11 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     prefetch_tensormap(&tm_a);
     prefetch_tensormap(&tm_b0);
     prefetch_tensormap(&tm_b1);
+    if (kPair) {
+      prefetch_tensormap(&ts_a);
+      prefetch_tensormap(&ts_b0);
+      prefetch_tensormap(&ts_b1);
+    }
   }
   if (warp == 2) {
     tmem_alloc(smem_u32(&bars->tmem_base), kTmemCols);
@@ -230,412 +682,72 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   pdl_wait();                              // set-up above overlaps the tail of the kernel before this one
   const int n_mtiles = a.tiles[0].x;
   const ItemPlan plan = plan_items<TR::kGateUp>(a, n_mtiles);
-  const int n_items = plan.n_items, n_whole = plan.n_whole;
+  const int n_whole = plan.n_whole;
+  int n_mt_s = 0, n_shared = 0;
+  if (kPair) {
+    n_mt_s = as.tiles[0].x;
+    n_shared = n_mt_s * as.n_ntiles * (TR::kGateUp ? 1 : as.k_splits);
+  }
+  const int n_items = plan.n_items + n_shared;
+  // item -> its number among the items of its kind
+  auto is_shared = [&](int item) { return kPair && (TR::kGateUp ? item < n_shared : item >= plan.n_items); };
+  auto shared_no = [&](int item) { return TR::kGateUp ? item : item - plan.n_items; };
+  auto routed_no = [&](int item) { return TR::kGateUp && kPair ? item - n_shared : item; };
 
   if (warp == 0) {
     // ---------------------------------------------------------------- token-operand producer
     if (lane == 0) {
-      uint32_t stage = 0, phase = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-        int4 tile; int n_tile, half;
-        decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
-        const int width = half < 0 ? a.bn : 128;
-        const int b_row = (a.b_rows_per_expert ? tile.x * a.b_rows_per_expert : 0) +
-                          n_tile * (TR::kGateUp ? a.bn / 2 : a.bn) + (half > 0 ? 128 : 0);
-        int kb, ke;
-        item_k_range<TR::kGateUp>(a, item, kb, ke);
-        for (int ks = kb; ks < ke; ++ks) {
-          if (!(ok = mbar_wait(smem_u32(&bars->empty[stage]), phase ^ 1, abort_flag))) break;
-          const uint32_t bar = smem_u32(&bars->full_a[stage]);
-          if (TR::kTernary) {
-            mbar_expect_tx(bar, kStageA);
-            tma_load_2d(sA + stage * kStageA, &tm_a, ks * 128, tile.y, bar);
-          } else if (TR::kRtn) {
-            mbar_expect_tx(bar, kStageA);
-            tma_load_2d(sA + stage * kStageA, &tm_a, ks * 64, tile.y, bar);
-          } else {
-            mbar_expect_tx(bar, kStageA + width * 128);
-            tma_load_2d(sA + stage * kStageA, &tm_a, ks * 64, tile.y, bar);
-            if (TR::kGateUp) {
-              tma_load_2d(sB + stage * kStageB, &tm_b0, ks * 64, b_row, bar);
-              tma_load_2d(sB + stage * kStageB + 128 * 128, &tm_b1, ks * 64, b_row, bar);
-            } else {
-              tma_load_2d(sB + stage * kStageB, &tm_b0, ks * 64, b_row, bar);
-              if (width > 128) tma_load_2d(sB + stage * kStageB + 128 * 128, &tm_b1, ks * 64, b_row + 128, bar);
-            }
-          }
-          if (++stage == S) { stage = 0; phase ^= 1; }
-        }
+      RingPos p;
+      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const bool ok = is_shared(item)
+            ? load_operands<kS, S>(ts_a, ts_b0, ts_b1, as, shared_no(item), n_mt_s, n_shared, sA, sB, bars, p)
+            : load_operands<MODE, S>(tm_a, tm_b0, tm_b1, a, routed_no(item), n_mtiles, n_whole, sA, sB, bars, p);
+        if (!ok) break;
       }
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- packed-weight producer
     if (TR::kUnpack && lane == 0) {
-      constexpr int kRB = TR::kCodeRowBytes;
-      uint32_t stage = 0, phase = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-        int4 tile; int n_tile, half;
-        decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
-        const int width = half < 0 ? a.bn : 128;
-        const int b_row = tile.x * a.b_rows_per_expert + n_tile * (TR::kGateUp ? a.bn / 2 : a.bn) + (half > 0 ? 128 : 0);
-        int kb, ke;
-        item_k_range<TR::kGateUp>(a, item, kb, ke);
-        for (int ks = kb; ks < ke; ++ks) {
-          if (!(ok = mbar_wait(smem_u32(&bars->empty_p[stage]), phase ^ 1, abort_flag))) break;
-          const uint32_t bar = smem_u32(&bars->full_p[stage]);
-          mbar_expect_tx(bar, width * kRB);
-          const uint32_t dst = sP + stage * TR::kStageP;
-          if (TR::kGateUp) {
-            tma_load_2d(dst, &tm_b0, ks * kRB, b_row, bar);
-            tma_load_2d(dst + 128 * kRB, &tm_b1, ks * kRB, b_row, bar);
-          } else {
-            tma_load_2d(dst, &tm_b0, ks * kRB, b_row, bar);
-            if (width > 128) tma_load_2d(dst + 128 * kRB, &tm_b1, ks * kRB, b_row + 128, bar);
-          }
-          if (++stage == TR::kStagesP) { stage = 0; phase ^= 1; }
-        }
+      RingPos p;
+      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        bool ok = true;
+        if (!is_shared(item)) ok = load_codes<MODE, kStagesP, kStageP>(tm_b0, tm_b1, a, routed_no(item), n_mtiles, n_whole, sP, bars, p);
+        else if (ModeTraits<kS>::kUnpack) ok = load_codes<kS, kStagesP, kStageP>(ts_b0, ts_b1, as, shared_no(item), n_mt_s, n_shared, sP, bars, p);
+        if (!ok) break;
       }
     }
   } else if (warp == 2) {
     // ---------------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      const uint32_t idesc_whole = TR::kTernary ? make_idesc(2, 1, 0, kBM, (uint32_t)a.bn)     // s32 += s8 * u8
-                                                : make_idesc(1, 1, 1, kBM, (uint32_t)a.bn);    // f32 += bf16 * bf16
-      const uint32_t idesc_half = TR::kTernary ? make_idesc(2, 1, 0, kBM, 128u) : make_idesc(1, 1, 1, kBM, 128u);
-      uint32_t stage = 0, phase = 0;
+      RingPos p;
       int local = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x, ++local) {
-        const int buf = local & 1;
-        const uint32_t use = (uint32_t)(local >> 1);
-        if (!(ok = mbar_wait(smem_u32(&bars->tmem_empty[buf]), (use & 1) ^ 1, abort_flag))) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + buf * 256;
-        const uint32_t idesc = (!TR::kGateUp && item >= n_whole) ? idesc_half : idesc_whole;
-        int kb, ke;
-        item_k_range<TR::kGateUp>(a, item, kb, ke);
-        for (int ks = kb; ks < ke; ++ks) {
-          if (!(ok = mbar_wait(smem_u32(&bars->full_a[stage]), phase, abort_flag))) break;
-          if (TR::kUnpack)
-            if (!(ok = mbar_wait(smem_u32(&bars->full_u[stage]), phase, abort_flag))) break;
-          tc_fence_after();
-          const uint64_t da = smem_desc_sw128(sA + stage * kStageA);
-          const uint64_t db = smem_desc_sw128(sB + stage * kStageB);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t acc = (ks > kb || j > 0) ? 1u : 0u;
-            if (TR::kTernary) mma_i8(d_tmem, da + 2 * j, db + 2 * j, idesc, acc);
-            else mma_f16(d_tmem, da + 2 * j, db + 2 * j, idesc, acc);
-          }
-          mma_commit(smem_u32(&bars->empty[stage]));
-          if (++stage == S) { stage = 0; phase ^= 1; }
-        }
-        if (ok) mma_commit(smem_u32(&bars->tmem_full[buf]));
+      for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++local) {
+        const bool ok = is_shared(item)
+            ? issue_mmas<kS, S, TR::kUnpack>(as, shared_no(item), n_shared, local, tmem_base, sA, sB, bars, p)
+            : issue_mmas<MODE, S, TR::kUnpack>(a, routed_no(item), n_whole, local, tmem_base, sA, sB, bars, p);
+        if (!ok) break;
       }
     }
   } else if (warp >= 4 && warp < 12) {
     // ---------------------------------------------------------------- code unpackers
-    // (2-bit -> int8 for the ternary experts; int8 / 4-bit -> bf16 for an RTN-coded shared expert)
-    // group 0 (warps 4-7) expands the even pipeline steps, group 1 (warps 8-11) the odd ones
     if (TR::kUnpack) {
       const int group = (warp - 4) >> 2;
-      const int tid = (threadIdx.x - 128) & 127;
-      uint32_t stage = 0, phase = 0, pstage = 0, pphase = 0, step = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-        // chunks of 16 code bytes, spread over 128 threads
-        const int n_chunks = ((!TR::kGateUp && item >= n_whole) ? 128 : a.bn) * (TR::kCodeRowBytes / 16);
-        int kb, ke;
-        item_k_range<TR::kGateUp>(a, item, kb, ke);
-        for (int ks = kb; ks < ke; ++ks, ++step) {
-          if ((step & 1u) == (uint32_t)group) {
-            ok = mbar_wait(smem_u32(&bars->full_p[pstage]), pphase, abort_flag) &&
-                 mbar_wait(smem_u32(&bars->empty[stage]), phase ^ 1, abort_flag);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            const uint8_t* src = genP + pstage * TR::kStageP;
-            uint8_t* dst = genB + stage * kStageB;
-            // batches of four chunks per thread, all loads of a batch ahead of its conversions
-            for (int c0 = tid; c0 < n_chunks; c0 += 128 * 4) {
-              uint4 wv[4];
-#pragma unroll
-              for (int b = 0; b < 4; ++b) {
-                const int c = c0 + b * 128;
-                if (c < n_chunks) wv[b] = *reinterpret_cast<const uint4*>(src + c * 16);
-              }
-#pragma unroll
-              for (int b = 0; b < 4; ++b) {
-                const int c = c0 + b * 128;
-                if (c >= n_chunks) break;
-                const uint32_t pw[4] = {wv[b].x, wv[b].y, wv[b].z, wv[b].w};
-                if (TR::kRtnBits == 8) {
-                  // 16 int8 codes -> two 16-byte pieces of 8 bf16 each
-                  const int r = c >> 2, quarter = c & 3;
-                  uint8_t* row = dst + (r >> 3) * 1024 + (r & 7) * 128;
-                  uint32_t e[8];
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) s8x4_to_bf16x2(pw[j], e[2 * j], e[2 * j + 1]);
-                  *reinterpret_cast<uint4*>(row + (((quarter * 2) ^ (r & 7)) << 4)) = make_uint4(e[0], e[1], e[2], e[3]);
-                  *reinterpret_cast<uint4*>(row + (((quarter * 2 + 1) ^ (r & 7)) << 4)) = make_uint4(e[4], e[5], e[6], e[7]);
-                } else {
-                  const int r = c >> 1, half = c & 1;
-                  uint8_t* row = dst + (r >> 3) * 1024 + (r & 7) * 128;
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    uint4 o;
-                    if (TR::kRtnBits == 4) {
-                      // 8 four-bit codes -> one 16-byte piece of 8 bf16
-                      uint32_t e[4];
-                      u4x8_to_bf16x2(pw[j], e);
-                      o = make_uint4(e[0], e[1], e[2], e[3]);
-                    } else {
-                      o.x = pw[j] & 0x03030303u;
-                      o.y = (pw[j] >> 2) & 0x03030303u;
-                      o.z = (pw[j] >> 4) & 0x03030303u;
-                      o.w = (pw[j] >> 6) & 0x03030303u;
-                    }
-                    *reinterpret_cast<uint4*>(row + (((half * 4 + j) ^ (r & 7)) << 4)) = o;
-                  }
-                }
-              }
-            }
-            fence_proxy_async_smem();                // generic-proxy writes -> visible to the MMA
-            __syncwarp();
-            if (lane == 0) {
-              mbar_arrive(smem_u32(&bars->full_u[stage]));
-              mbar_arrive(smem_u32(&bars->empty_p[pstage]));
-            }
-          }
-          if (++stage == S) { stage = 0; phase ^= 1; }
-          if (++pstage == TR::kStagesP) { pstage = 0; pphase ^= 1; }
-        }
+      RingPos p, q;
+      uint32_t step = 0;
+      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const bool ok = is_shared(item)
+            ? expand_codes<kS, S, kStagesP, kStageP>(as, shared_no(item), n_shared, group, genB, genP, bars, p, q, step)
+            : expand_codes<MODE, S, kStagesP, kStageP>(a, routed_no(item), n_whole, group, genB, genP, bars, p, q, step);
+        if (!ok) break;
       }
     }
   } else if (warp >= 12) {
     // ---------------------------------------------------------------- epilogue
-    const int q = warp & 3;                          // TMEM lane quarter this warp may read
-    const int chalf = (warp - 12) >> 2;              // which half of the tile's columns
-    const int r_in_tile = q * 32 + lane;
     int local = 0;
-    bool ok = true;
-    for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x, ++local) {
-      int4 tile; int n_tile, half;
-      decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
-      int kb_, ke_;
-      const int split = item_k_range<TR::kGateUp>(a, item, kb_, ke_);
-      const int buf = local & 1;
-      const uint32_t use = (uint32_t)(local >> 1);
-      ok = mbar_wait(smem_u32(&bars->tmem_full[buf]), use & 1, abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++local) {
+      const bool ok = is_shared(item) ? write_out<kS>(as, shared_no(item), n_mt_s, n_shared, local, tmem_base, genE, bars)
+                                      : write_out<MODE>(a, routed_no(item), n_mtiles, n_whole, local, tmem_base, genE, bars);
       if (!ok) break;
-      tc_fence_after();
-      const bool row_ok = r_in_tile < tile.z;
-      const int64_t row = int64_t(tile.y) + r_in_tile;
-      const uint32_t t_row = tmem_base + (uint32_t(q * 32) << 16) + buf * 256;
-      float c0 = 0.f, c1 = 0.f;
-      int rs = 0;
-      if (TR::kTernary && row_ok) {
-        const float beta = fmaxf(a.beta[row], kEpsScale);
-        rs = a.rowsum[row];
-        c0 = dequant_scale(a.alpha0[tile.x], beta);
-        if (TR::kGateUp) c1 = dequant_scale(a.alpha1[tile.x], beta);
-      }
-      if (TR::kGateUp) {
-        const int col0 = n_tile * 128;
-        const bool row_fast = __fmul_rn(c0, c1) > 1e-12f;
-        const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;
-        float hmax = 0.0f;                           // max |h| (before the bf16 rounding, which is monotonic)
-        constexpr int kCols = TR::kEpiCols, kPitch = TR::kEpiPitch;
-        constexpr int kLanesPerRow = kCols * 2 / 16, kRowsPerStore = 32 / kLanesPerRow;
-        uint8_t* stg = genE + (warp - 12) * 32 * kPitch;
-#pragma unroll 1
-        for (int cr = chalf * 64; cr < chalf * 64 + 64; cr += kCols) {
-#pragma unroll 1
-          for (int c = cr; c < cr + kCols; c += 16) {
-            uint32_t rg[16], ru[16];
-            tmem_ld_32x32b_x16(t_row + c, rg);
-            tmem_ld_32x32b_x16(t_row + 128 + c, ru);
-            tmem_wait_ld();
-            if (row_ok) {
-              float hv[16];
-              if (TR::kTernary) {
-                uint32_t redo_mask = 0u;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                  bool redo;
-                  hv[j] = glu_h_fast_biased(rg[j], ru[j], acc_bias, c0, c1, redo);
-                  if (redo) redo_mask |= 1u << j;
-                }
-                if (!row_fast) redo_mask = 0xFFFFu;
-                if (redo_mask) {                     // mostly one element: look at four at a time
-#pragma unroll
-                  for (int j0 = 0; j0 < 16; j0 += 4)
-                    if ((redo_mask >> j0) & 0xFu) {
-#pragma unroll
-                      for (int j = j0; j < j0 + 4; ++j)
-                        if ((redo_mask >> j) & 1u) hv[j] = glu_h_rare((int)rg[j] - rs, (int)ru[j] - rs, c0, c1);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) hmax = fmaxf(hmax, fabsf(hv[j]));
-              } else if (TR::kRtn || a.alpha0 != nullptr) {
-                // RTN-coded shared expert (codes expanded here, or beforehand): row scales of the
-                // gate and up matrices = scales of this tile's output columns
-                const float4* sgp = reinterpret_cast<const float4*>(a.alpha0 + col0 + c);
-                const float4* sup = reinterpret_cast<const float4*>(a.alpha1 + col0 + c);
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                  const float4 sg = __ldg(sgp + v), su = __ldg(sup + v);
-                  const float sgv[4] = {sg.x, sg.y, sg.z, sg.w}, suv[4] = {su.x, su.y, su.z, su.w};
-#pragma unroll
-                  for (int u = 0; u < 4; ++u) {
-                    const float g = __uint_as_float(rg[4 * v + u]) * sgv[u];
-                    hv[4 * v + u] = __uint_as_float(ru[4 * v + u]) * suv[u] * silu_fast(g);
-                  }
-                }
-              } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                  const float g = __uint_as_float(rg[j]);
-                  hv[j] = __uint_as_float(ru[j]) * silu_fast(g);
-                }
-              }
-              uint32_t packed[8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) packed[j] = pack_bf16x2(hv[2 * j], hv[2 * j + 1]);
-              if (TR::kTernary) {
-                // the thread's 16 bf16 values are one 32-byte sector of its row: one store
-                st_global_v8(reinterpret_cast<uint16_t*>(a.out) + row * a.n_out + col0 + c, packed[0], packed[1], packed[2],
-                             packed[3], packed[4], packed[5], packed[6], packed[7]);
-              } else {
-                uint4* sdst = reinterpret_cast<uint4*>(stg + lane * kPitch + (c - cr) * 2);
-                sdst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                sdst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-              }
-              if (TR::kTernary && a.tap0) {
-                int4* t0 = reinterpret_cast<int4*>(a.tap0 + row * a.n_out + col0 + c);
-                int4* t1 = reinterpret_cast<int4*>(a.tap1 + row * a.n_out + col0 + c);
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                  t0[v] = make_int4((int)rg[4 * v] - rs, (int)rg[4 * v + 1] - rs, (int)rg[4 * v + 2] - rs, (int)rg[4 * v + 3] - rs);
-                  t1[v] = make_int4((int)ru[4 * v] - rs, (int)ru[4 * v + 1] - rs, (int)ru[4 * v + 2] - rs, (int)ru[4 * v + 3] - rs);
-                }
-              }
-            }
-          }
-          if (!TR::kTernary) {
-            __syncwarp();
-            // the warp's 32 rows x kCols columns leave as whole row segments (kCols * 2 bytes each)
-#pragma unroll
-            for (int r0 = 0; r0 < 32; r0 += kRowsPerStore) {
-              const int r = r0 + lane / kLanesPerRow, piece = lane % kLanesPerRow;
-              if (q * 32 + r < tile.z) {
-                const uint4 v = *reinterpret_cast<const uint4*>(stg + r * kPitch + piece * 16);
-                uint16_t* orow = reinterpret_cast<uint16_t*>(a.out) + (int64_t(tile.y) + q * 32 + r) * a.n_out + col0 + cr;
-                reinterpret_cast<uint4*>(orow)[piece] = v;
-              }
-            }
-            __syncwarp();
-          }
-        }
-        // bits of non-negative floats order like unsigned integers; bf16_rn(max) = max(bf16_rn)
-        if (TR::kTernary && row_ok && a.beta_out_bits) {
-          const uint32_t hb = f32_to_bf16_bits(hmax) << 16;
-          if (hb) atomicMax(a.beta_out_bits + row, hb);
-        }
-      } else {
-        const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;   // see glu_h_fast_biased
-        const int width = half < 0 ? a.bn : 128;
-        const int col0 = n_tile * a.bn + (half > 0 ? 128 : 0);
-        const int cbeg = chalf * (width / 2), cend = cbeg + width / 2;
-        const bool combine = !TR::kTernary && a.comb_out != nullptr;
-        float cw[MOTE_MAX_TOPK];
-        const float* cy[MOTE_MAX_TOPK];
-        if (combine && row_ok) {
-#pragma unroll
-          for (int j = 0; j < MOTE_MAX_TOPK; ++j)
-            if (j < a.comb_k) {
-              cw[j] = a.comb_w[row * a.comb_k + j];
-              cy[j] = a.comb_y + int64_t(a.comb_perm[row * a.comb_k + j]) * a.n_out + col0;
-            }
-        }
-#pragma unroll 1
-        for (int c = cbeg; c < cend; c += 16) {
-          uint32_t ra[16];
-          tmem_ld_32x32b_x16(t_row + c, ra);
-          tmem_wait_ld();
-          if (row_ok) {
-            float o[16];
-#pragma unroll
-            for (int v = 0; v < 16; ++v)
-              o[v] = TR::kTernary ? __fmul_rn(__fsub_rn(__uint_as_float(ra[v] + acc_bias), kMagic), c0)   // fl32(acc - rs) * c0
-                                  : __uint_as_float(ra[v]);
-            if (TR::kRtn || (!TR::kTernary && a.alpha0 != nullptr)) {
-              const float4* sp = reinterpret_cast<const float4*>(a.alpha0 + col0 + c);
-#pragma unroll
-              for (int v = 0; v < 4; ++v) {
-                const float4 sc = __ldg(sp + v);
-                o[4 * v] *= sc.x; o[4 * v + 1] *= sc.y; o[4 * v + 2] *= sc.z; o[4 * v + 3] *= sc.w;
-              }
-            }
-            if (a.out) {
-              float* dst = reinterpret_cast<float*>(a.out) + split * a.split_stride + row * a.n_out + col0 + c;
-#pragma unroll
-              for (int v = 0; v < 2; ++v)
-                st_global_v8(dst + 8 * v, __float_as_uint(o[8 * v]), __float_as_uint(o[8 * v + 1]), __float_as_uint(o[8 * v + 2]),
-                             __float_as_uint(o[8 * v + 3]), __float_as_uint(o[8 * v + 4]), __float_as_uint(o[8 * v + 5]),
-                             __float_as_uint(o[8 * v + 6]), __float_as_uint(o[8 * v + 7]));
-            }
-            if (TR::kTernary && a.tap0) {
-              int4* t0 = reinterpret_cast<int4*>(a.tap0 + row * a.n_out + col0 + c);
-#pragma unroll
-              for (int v = 0; v < 4; ++v)
-                t0[v] = make_int4((int)ra[4 * v] - rs, (int)ra[4 * v + 1] - rs, (int)ra[4 * v + 2] - rs, (int)ra[4 * v + 3] - rs);
-            }
-            if (combine) {
-              // fp32, slots in ascending j, then the residual, one bf16 rounding
-#pragma unroll
-              for (int j = 0; j < MOTE_MAX_TOPK; ++j)
-                if (j < a.comb_k) {
-#pragma unroll
-                  for (int v = 0; v < 2; ++v) {
-                    uint32_t yv[8];
-                    ld_global_v8(cy[j] + c + 8 * v, yv);
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) o[8 * v + u] = fmaf(cw[j], __uint_as_float(yv[u]), o[8 * v + u]);
-                  }
-                }
-              if (a.comb_res) {
-                uint32_t rw[8];
-                if (a.comb_wide) {
-                  ld_global_v8(a.comb_res + row * a.n_out + col0 + c, rw);
-                } else {
-                  const uint4* rp = reinterpret_cast<const uint4*>(a.comb_res + row * a.n_out + col0 + c);
-                  const uint4 r0 = rp[0], r1 = rp[1];
-                  rw[0] = r0.x; rw[1] = r0.y; rw[2] = r0.z; rw[3] = r0.w; rw[4] = r1.x; rw[5] = r1.y; rw[6] = r1.z; rw[7] = r1.w;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) { o[2 * u] += bf16_lo(rw[u]); o[2 * u + 1] += bf16_hi(rw[u]); }
-              }
-              uint32_t pk[8];
-#pragma unroll
-              for (int v = 0; v < 8; ++v) pk[v] = f32_to_bf16_bits(o[2 * v]) | (f32_to_bf16_bits(o[2 * v + 1]) << 16);
-              if (a.comb_wide) {
-                st_global_v8(a.comb_out + row * a.n_out + col0 + c, pk[0], pk[1], pk[2], pk[3], pk[4], pk[5], pk[6], pk[7]);
-              } else {
-                uint4* od = reinterpret_cast<uint4*>(a.comb_out + row * a.n_out + col0 + c);
-                od[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                od[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-              }
-            }
-          }
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->tmem_empty[buf]));
     }
   }
 
@@ -649,6 +761,20 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     tmem_dealloc(tmem_base, kTmemCols);
   }
   if (threadIdx.x == 0) report_abort(abort_flag, a.status);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kThreads, 1)
+umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
+                 const __grid_constant__ CUtensorMap tm_b1, const UmmaArgs a) {
+  umma_cta<MODE, -1>(tm_a, tm_b0, tm_b1, a, tm_a, tm_b0, tm_b1, a);
+}
+template <int MODE, int SMODE>
+__global__ void __launch_bounds__(kThreads, 1)
+umma_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
+                 const __grid_constant__ CUtensorMap tm_b1, const UmmaArgs a, const __grid_constant__ CUtensorMap ts_a,
+                 const __grid_constant__ CUtensorMap ts_b0, const __grid_constant__ CUtensorMap ts_b1, const UmmaArgs as) {
+  umma_cta<MODE, SMODE>(tm_a, tm_b0, tm_b1, a, ts_a, ts_b0, ts_b1, as);
 }
 
 // One CTA that runs the GEMM kernels' bounded wait to its limit: an mbarrier nothing ever arrives
@@ -733,11 +859,14 @@ static mote_status_t launch_umma(const CUtensorMap& ta, const CUtensorMap& tb0, 
   return MOTE_OK;
 }
 
-mote_status_t launch_ternary_umma(const TernaryGemmArgs& g, bool gateup, const int4* tiles, int max_mtiles,
-                                  const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status,
-                                  cudaStream_t stream, bool pdl) {
-  if (g.P == 0) return MOTE_OK;
+// Tensor maps and arguments of one GEMM.
+struct GemmSetup {
   CUtensorMap ta, tb0, tb1;
+  UmmaArgs a{};
+};
+
+static bool setup_ternary(GemmSetup& u, const TernaryGemmArgs& g, bool gateup, const int4* tiles, int max_mtiles,
+                          const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status) {
   int bn = gateup ? 256 : pick_bn(g.N);
   // a down projection with few row tiles: 128-wide tiles double the items (the weights are the
   // traffic here, and they are read once either way)
@@ -745,17 +874,15 @@ mote_status_t launch_ternary_umma(const TernaryGemmArgs& g, bool gateup, const i
     const int sms = device_sm_count();
     if (max_mtiles * (g.N / bn) * 2 <= sms) bn = 128;
   }
-  if (!make_map_2d(&ta, g.qa, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.P, (uint64_t)g.K, 128, 128,
-                   CU_TENSOR_MAP_SWIZZLE_128B))
-    return MOTE_ERR_CUDA;
-  if (!make_map_2d(&tb0, g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N, (uint64_t)g.K / 4, 128, 32,
-                   CU_TENSOR_MAP_SWIZZLE_NONE))
-    return MOTE_ERR_CUDA;
-  // second map: the up matrix (gate/up), or the rows beyond 128 of a down tile
-  if (!make_map_2d(&tb1, gateup ? g.w1 : g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N,
+  // second weight map: the up matrix (gate/up), or the rows beyond 128 of a down tile
+  if (!make_map_2d(&u.ta, g.qa, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.P, (uint64_t)g.K, 128, 128,
+                   CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_map_2d(&u.tb0, g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N, (uint64_t)g.K / 4, 128, 32,
+                   CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !make_map_2d(&u.tb1, gateup ? g.w1 : g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N,
                    (uint64_t)g.K / 4, (gateup || bn <= 128) ? 128 : bn - 128, 32, CU_TENSOR_MAP_SWIZZLE_NONE))
-    return MOTE_ERR_CUDA;
-  UmmaArgs a{};
+    return false;
+  UmmaArgs& a = u.a;
   a.tiles = tiles;
   a.n_ntiles = gateup ? g.N / 128 : g.N / bn;
   a.k_steps = g.K / 128;
@@ -769,9 +896,18 @@ mote_status_t launch_ternary_umma(const TernaryGemmArgs& g, bool gateup, const i
   a.tap0 = g.acc0_tap; a.tap1 = g.acc1_tap;
   a.beta_out_bits = gateup ? beta_out_bits : nullptr;
   a.status = status;
-  const int max_items = max_mtiles * a.n_ntiles;
-  return gateup ? launch_umma<MODE_T_GATEUP>(ta, tb0, tb1, a, max_items, stream, pdl)
-                : launch_umma<MODE_T_DOWN>(ta, tb0, tb1, a, max_items, stream, pdl);
+  return true;
+}
+
+mote_status_t launch_ternary_umma(const TernaryGemmArgs& g, bool gateup, const int4* tiles, int max_mtiles,
+                                  const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status,
+                                  cudaStream_t stream, bool pdl) {
+  if (g.P == 0) return MOTE_OK;
+  GemmSetup u;
+  if (!setup_ternary(u, g, gateup, tiles, max_mtiles, rowsum, beta_out_bits, status)) return MOTE_ERR_CUDA;
+  const int max_items = max_mtiles * u.a.n_ntiles;
+  return gateup ? launch_umma<MODE_T_GATEUP>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl)
+                : launch_umma<MODE_T_DOWN>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl);
 }
 
 // K splits of the shared down projection: with few row tiles its T x N output has too few tiles to
@@ -787,36 +923,32 @@ int shared_down_k_splits(int64_t T, int N, int K) {
   return (int)std::max<int64_t>(splits, 1);
 }
 
-mote_status_t launch_shared_umma(const void* act, const SharedMat& w0, const SharedMat& w1, int bits, bool gateup,
-                                 int64_t T, int K, int N, void* out, const int4* tiles, int max_mtiles,
-                                 uint32_t* status, const CombineArgs* comb, cudaStream_t stream, bool pdl,
-                                 int k_splits) {
-  if (T == 0) return MOTE_OK;
-  if (k_splits > 1 && (gateup || comb || !out)) return MOTE_ERR_SHAPE;
-  CUtensorMap ta, tb0, tb1;
+static bool setup_shared(GemmSetup& u, const void* act, const SharedMat& w0, const SharedMat& w1, int bits, bool gateup,
+                         int64_t T, int K, int N, void* out, const int4* tiles, uint32_t* status, const CombineArgs* comb,
+                         int k_splits) {
   const int bn = gateup ? 256 : pick_bn(N);
   const uint32_t rows1 = (gateup || bn <= 128) ? 128 : bn - 128;
-  if (!make_map_2d(&ta, act, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)T, (uint64_t)K, 128, 64,
+  if (!make_map_2d(&u.ta, act, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)T, (uint64_t)K, 128, 64,
                    CU_TENSOR_MAP_SWIZZLE_128B))
-    return MOTE_ERR_CUDA;
+    return false;
   const void* wb1 = gateup ? w1.w : w0.w;
   if (bits == 16) {
-    if (!make_map_2d(&tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)N, (uint64_t)K, 128, 64,
+    if (!make_map_2d(&u.tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)N, (uint64_t)K, 128, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_2d(&tb1, wb1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)N, (uint64_t)K, rows1, 64,
+        !make_map_2d(&u.tb1, wb1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)N, (uint64_t)K, rows1, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B))
-      return MOTE_ERR_CUDA;
+      return false;
   } else {
     // code rows as bytes: K (int8) or K/2 (4-bit) per row, 64 reduction elements per pipeline stage
     const uint64_t row_bytes = bits == 8 ? (uint64_t)K : (uint64_t)K / 2;
     const uint32_t box = bits == 8 ? 64 : 32;
-    if (!make_map_2d(&tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, row_bytes, 128, box,
+    if (!make_map_2d(&u.tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, row_bytes, 128, box,
                      CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !make_map_2d(&tb1, wb1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, row_bytes, rows1, box,
+        !make_map_2d(&u.tb1, wb1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, row_bytes, rows1, box,
                      CU_TENSOR_MAP_SWIZZLE_NONE))
-      return MOTE_ERR_CUDA;
+      return false;
   }
-  UmmaArgs a{};
+  UmmaArgs& a = u.a;
   a.tiles = tiles;
   a.n_ntiles = gateup ? N / 128 : N / bn;
   a.k_steps = K / 64;
@@ -835,15 +967,63 @@ mote_status_t launch_shared_umma(const void* act, const SharedMat& w0, const Sha
     a.comb_k = comb->k;
     a.comb_wide = ((reinterpret_cast<uintptr_t>(comb->out) | reinterpret_cast<uintptr_t>(comb->residual)) & 31u) == 0;
   }
+  return true;
+}
+
+mote_status_t launch_shared_umma(const void* act, const SharedMat& w0, const SharedMat& w1, int bits, bool gateup,
+                                 int64_t T, int K, int N, void* out, const int4* tiles, int max_mtiles,
+                                 uint32_t* status, const CombineArgs* comb, cudaStream_t stream, bool pdl,
+                                 int k_splits) {
+  if (T == 0) return MOTE_OK;
+  if (k_splits > 1 && (gateup || comb || !out)) return MOTE_ERR_SHAPE;
+  GemmSetup u;
+  if (!setup_shared(u, act, w0, w1, bits, gateup, T, K, N, out, tiles, status, comb, k_splits)) return MOTE_ERR_CUDA;
+  const UmmaArgs& a = u.a;
   const int max_items = max_mtiles * a.n_ntiles * a.k_splits;
   if (bits == 8)
-    return gateup ? launch_umma<MODE_Q8_GATEUP>(ta, tb0, tb1, a, max_items, stream, pdl)
-                  : launch_umma<MODE_Q8_DOWN>(ta, tb0, tb1, a, max_items, stream, pdl);
+    return gateup ? launch_umma<MODE_Q8_GATEUP>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl)
+                  : launch_umma<MODE_Q8_DOWN>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl);
   if (bits == 4)
-    return gateup ? launch_umma<MODE_Q4_GATEUP>(ta, tb0, tb1, a, max_items, stream, pdl)
-                  : launch_umma<MODE_Q4_DOWN>(ta, tb0, tb1, a, max_items, stream, pdl);
-  return gateup ? launch_umma<MODE_B_GATEUP>(ta, tb0, tb1, a, max_items, stream, pdl)
-                : launch_umma<MODE_B_DOWN>(ta, tb0, tb1, a, max_items, stream, pdl);
+    return gateup ? launch_umma<MODE_Q4_GATEUP>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl)
+                  : launch_umma<MODE_Q4_DOWN>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl);
+  return gateup ? launch_umma<MODE_B_GATEUP>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl)
+                : launch_umma<MODE_B_DOWN>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl);
+}
+
+template <int MODE, int SMODE>
+static mote_status_t launch_pair(const GemmSetup& r, const GemmSetup& sh, int max_items, cudaStream_t stream, bool pdl) {
+  constexpr size_t smem = PairTraits<MODE, SMODE>::kSmem;
+  static PerDeviceOnce attr_once;                  // one per pair
+  MOTE_CUDA_OK(set_max_dynamic_smem(attr_once, umma_pair_kernel<MODE, SMODE>, (int)smem));
+  const int grid = std::max(1, std::min(device_sm_count(), max_items));
+  if (pdl)
+    MOTE_CUDA_OK(launch_pdl(umma_pair_kernel<MODE, SMODE>, dim3(grid), dim3(kThreads), smem, stream, r.ta, r.tb0, r.tb1, r.a,
+                            sh.ta, sh.tb0, sh.tb1, sh.a));
+  else
+    umma_pair_kernel<MODE, SMODE><<<grid, kThreads, smem, stream>>>(r.ta, r.tb0, r.tb1, r.a, sh.ta, sh.tb0, sh.tb1, sh.a);
+  ++g_launch_count;
+  MOTE_LAUNCH_OK();
+  return MOTE_OK;
+}
+
+mote_status_t launch_umma_pair(const TernaryGemmArgs& g, bool gateup, const int4* tiles_routed, int max_mtiles_routed,
+                               const int32_t* rowsum, uint32_t* beta_out_bits, const void* act, const SharedMat& w0,
+                               const SharedMat& w1, int bits, int64_t T, void* out, const int4* tiles_shared,
+                               int max_mtiles_shared, uint32_t* status, cudaStream_t stream, bool pdl, int k_splits) {
+  if (g.P == 0) return MOTE_OK;
+  GemmSetup r, sh;
+  if (!setup_ternary(r, g, gateup, tiles_routed, max_mtiles_routed, rowsum, beta_out_bits, status) ||
+      !setup_shared(sh, act, w0, w1, bits, gateup, T, g.K, g.N, out, tiles_shared, status, nullptr, k_splits))
+    return MOTE_ERR_CUDA;
+  const int max_items = max_mtiles_routed * r.a.n_ntiles + max_mtiles_shared * sh.a.n_ntiles * sh.a.k_splits;
+  if (bits == 8)
+    return gateup ? launch_pair<MODE_T_GATEUP, MODE_Q8_GATEUP>(r, sh, max_items, stream, pdl)
+                  : launch_pair<MODE_T_DOWN, MODE_Q8_DOWN>(r, sh, max_items, stream, pdl);
+  if (bits == 4)
+    return gateup ? launch_pair<MODE_T_GATEUP, MODE_Q4_GATEUP>(r, sh, max_items, stream, pdl)
+                  : launch_pair<MODE_T_DOWN, MODE_Q4_DOWN>(r, sh, max_items, stream, pdl);
+  return gateup ? launch_pair<MODE_T_GATEUP, MODE_B_GATEUP>(r, sh, max_items, stream, pdl)
+                : launch_pair<MODE_T_DOWN, MODE_B_DOWN>(r, sh, max_items, stream, pdl);
 }
 
 }  // namespace mote

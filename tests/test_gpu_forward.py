@@ -211,6 +211,23 @@ def test_rtn_shared_expert(mote, d, f, E, k, T, kw, path, bits):
     check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
 
 
+@pytest.mark.parametrize("bits", [16, 8, 4])
+@pytest.mark.parametrize("d,f,E,k,T,kw", [
+    (128, 512, 2, 1, 33, {}),                             # the smallest: one row tile per kind, one pipeline step of gate/up
+    (896, 640, 4, 2, 129, dict(bias="zipf")),             # a second row tile of one row; 224-wide shared down tiles
+    (256, 4864, 16, 2, 64, dict(outlier_frac=0.01)),      # sixteen K splits, odd numbers of pipeline steps per split
+    (1536, 384, 8, 2, 333, dict(norm_topk=0)),            # more items than SMs: CTAs walk from one kind to the other
+    (2048, 512, 8, 1, 1000, {}),                          # the most row tiles: two K splits
+])
+def test_short_prefill_pairs_of_gemms(mote, d, f, E, k, T, kw, bits):
+    wl = synth.custom("pair", d, f, E, k, T, 5000 + d + f + T, **kw)
+    master, layer_or, layer_gpu = _setup(mote, wl, TENSOR)
+    if bits != 16:
+        layer_or = O.quantize_shared(layer_or, bits)
+        layer_gpu = layer_gpu.quantize_shared(bits)
+    check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
+
+
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("path", ALL)
 def test_rtn_shared_expert_c3_decode(mote, path, bits, c3_layers):
