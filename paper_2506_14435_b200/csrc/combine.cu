@@ -8,50 +8,63 @@
 
 namespace mote {
 
+// Its calls are short (a few hundred tokens; long prefills combine in the shared down GEMM's epilogue), so it is bound by
+// the latency of its loads and by how many are in flight: a thread owns four columns, not eight (twice the CTAs), and
+// asks for the partial sums eight at a time and for the expert rows ahead of them.
+__device__ __forceinline__ void add4(float (&acc)[4], const float4& a) { acc[0] += a.x; acc[1] += a.y; acc[2] += a.z; acc[3] += a.w; }
+
 __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ s, const float* __restrict__ y,
                                                       const float* __restrict__ w, const int32_t* __restrict__ perm,
                                                       const uint16_t* residual, int64_t T, int d, int k,
                                                       uint16_t* out, int n_partials) {
-  const int vec_per_row = d / 8;
+  constexpr int kBatch = 8, kEarly = 2;
+  const int vec_per_row = d / 4;
   const int64_t total = T * vec_per_row;
   pdl_wait();                            // no-op unless launched as a programmatic dependent
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
     const int64_t t = i / vec_per_row;
     const int v = (int)(i - t * vec_per_row);
-    float acc[8];
-    {
-      const float4* sp = reinterpret_cast<const float4*>(s + t * d + v * 8);
-      const float4 a = sp[0], b = sp[1];
-      acc[0] = a.x; acc[1] = a.y; acc[2] = a.z; acc[3] = a.w;
-      acc[4] = b.x; acc[5] = b.y; acc[6] = b.z; acc[7] = b.w;
-    }
-    for (int p = 1; p < n_partials; ++p) {           // partial sums of a K-split projection, in order
-      const float4* sp = reinterpret_cast<const float4*>(s + (int64_t(p) * T + t) * d + v * 8);
-      const float4 a = sp[0], b = sp[1];
-      acc[0] += a.x; acc[1] += a.y; acc[2] += a.z; acc[3] += a.w;
-      acc[4] += b.x; acc[5] += b.y; acc[6] += b.z; acc[7] += b.w;
+    float wj[kEarly];
+    float4 yj[kEarly];
+#pragma unroll
+    for (int j = 0; j < kEarly; ++j)
+      if (j < k) {
+        wj[j] = w[t * k + j];
+        yj[j] = *reinterpret_cast<const float4*>(y + int64_t(perm[t * k + j]) * d + v * 4);
+      }
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const float* sp = s + t * d + v * 4;
+    for (int p0 = 0; p0 < n_partials; p0 += kBatch) {   // partial sums of a K-split projection, in order
+      float4 sv[kBatch];
+#pragma unroll
+      for (int p = 0; p < kBatch; ++p)
+        if (p0 + p < n_partials) sv[p] = *reinterpret_cast<const float4*>(sp + int64_t(p0 + p) * T * d);
+#pragma unroll
+      for (int p = 0; p < kBatch; ++p) {
+        if (p0 + p == 0) { acc[0] = sv[0].x; acc[1] = sv[0].y; acc[2] = sv[0].z; acc[3] = sv[0].w; }
+        else if (p0 + p < n_partials) add4(acc, sv[p]);
+      }
     }
     for (int j = 0; j < k; ++j) {
-      const float wj = w[t * k + j];
-      const int64_t r = perm[t * k + j];
-      const float4* yp = reinterpret_cast<const float4*>(y + r * d + v * 8);
-      const float4 a = yp[0], b = yp[1];
-      acc[0] = fmaf(wj, a.x, acc[0]); acc[1] = fmaf(wj, a.y, acc[1]);
-      acc[2] = fmaf(wj, a.z, acc[2]); acc[3] = fmaf(wj, a.w, acc[3]);
-      acc[4] = fmaf(wj, b.x, acc[4]); acc[5] = fmaf(wj, b.y, acc[5]);
-      acc[6] = fmaf(wj, b.z, acc[6]); acc[7] = fmaf(wj, b.w, acc[7]);
+      float wv;
+      float4 a;
+      if (j < kEarly) {
+        wv = j == 0 ? wj[0] : wj[1];
+        a = j == 0 ? yj[0] : yj[1];
+      } else {
+        wv = w[t * k + j];
+        a = *reinterpret_cast<const float4*>(y + int64_t(perm[t * k + j]) * d + v * 4);
+      }
+      acc[0] = fmaf(wv, a.x, acc[0]); acc[1] = fmaf(wv, a.y, acc[1]);
+      acc[2] = fmaf(wv, a.z, acc[2]); acc[3] = fmaf(wv, a.w, acc[3]);
     }
     if (residual) {
-      const uint4 r = *reinterpret_cast<const uint4*>(residual + t * d + v * 8);
-      const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) { acc[2 * q] += bf16_lo(rw[q]); acc[2 * q + 1] += bf16_hi(rw[q]); }
+      const uint2 r = *reinterpret_cast<const uint2*>(residual + t * d + v * 4);
+      acc[0] += bf16_lo(r.x); acc[1] += bf16_hi(r.x); acc[2] += bf16_lo(r.y); acc[3] += bf16_hi(r.y);
     }
-    uint32_t o[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) o[q] = f32_to_bf16_bits(acc[2 * q]) | (f32_to_bf16_bits(acc[2 * q + 1]) << 16);
-    *reinterpret_cast<uint4*>(out + t * d + v * 8) = make_uint4(o[0], o[1], o[2], o[3]);
+    *reinterpret_cast<uint2*>(out + t * d + v * 4) =
+        make_uint2(f32_to_bf16_bits(acc[0]) | (f32_to_bf16_bits(acc[1]) << 16), f32_to_bf16_bits(acc[2]) | (f32_to_bf16_bits(acc[3]) << 16));
   }
 }
 
@@ -59,7 +72,7 @@ mote_status_t launch_combine(const float* s, const float* y, const float* w, con
                              const void* residual, int64_t T, int d, int k, void* out_bf16, cudaStream_t stream,
                              bool pdl, int n_partials) {
   if (T == 0) return MOTE_OK;
-  const int64_t total = T * (d / 8);
+  const int64_t total = T * (d / 4);
   const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, 148 * 16);
   if (pdl)
     MOTE_CUDA_OK(launch_pdl(combine_kernel, dim3(blocks), dim3(256), 0, stream, s, y, w, perm,
