@@ -361,8 +361,10 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
                          blockwise ? blk_hist : nullptr, stream, router_clears ? status : nullptr);
   if (st) return st;
   stage_mark(1, stream);
-  st = blockwise ? launch_dispatch_scan(blk_hist, n_blk, E, offsets, blk_base, tiles_routed, tiles_shared, T, stream)
-                 : launch_dispatch(topk_idx, P, E, offsets, perm, inv, tensor ? tiles_routed : nullptr,
+  const bool inline_scan = blockwise && n_blk <= kInlineScanBlocks;   // few blocks: done by the CTAs of Q_a(x)
+  st = inline_scan ? MOTE_OK
+       : blockwise ? launch_dispatch_scan(blk_hist, n_blk, E, offsets, blk_base, tiles_routed, tiles_shared, T, stream)
+                   : launch_dispatch(topk_idx, P, E, offsets, perm, inv, tensor ? tiles_routed : nullptr,
                                    tensor ? tiles_shared : nullptr, T, stream);
   if (st) return st;
   stage_mark(2, stream);
@@ -371,7 +373,12 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   qa.x = x; qa.T = T; qa.d = d; qa.ldx = d; qa.q = qx; qa.beta = beta_x; qa.rowsum = rowsum_x;
   qa.perm = perm; qa.k = k; qa.interleave = interleave;
   if (blockwise) {
-    qa.topk_idx = topk_idx; qa.blk_base = blk_base; qa.E = E; qa.n_blk = n_blk; qa.perm_out = perm; qa.inv_out = inv;
+    if (inline_scan) {
+      qa.blk_hist = blk_hist; qa.offsets_out = offsets; qa.tiles_routed = tiles_routed; qa.tiles_shared = tiles_shared;
+    } else {
+      qa.blk_base = blk_base;
+    }
+    qa.topk_idx = topk_idx; qa.E = E; qa.n_blk = n_blk; qa.perm_out = perm; qa.inv_out = inv;
     qa.zero_u32 = reinterpret_cast<uint32_t*>(beta_h); qa.zero_i32 = rowsum_h;
   }
   const bool pdl = blockwise;    // from here on every kernel is a programmatic dependent of the one before

@@ -20,12 +20,16 @@ struct QuantActArgs {
   // scatter variant with the block-wise dispatch: the destination row is derived here from the
   // top-k indices and the per-block bases, and written to perm_out / inv_out
   const int32_t* topk_idx; const int32_t* blk_base; int E; int n_blk;
+  // few blocks (n_blk <= kInlineScanBlocks, blk_base null): every CTA derives the bases from the router's block counts,
+  // and the first one writes the tables that launch_dispatch_scan would have written
+  const int32_t* blk_hist; int32_t* offsets_out; int4* tiles_routed; int4* tiles_shared;
   int32_t* perm_out; int32_t* inv_out;
   uint32_t* zero_u32; int32_t* zero_i32;   // optional [rows] arrays cleared at every destination row
   int k;
   int interleave;       // 1: store each unit of 16 codes k-interleaved
   int group;            // threads per row (set by the launcher)
 };
+constexpr int kInlineScanBlocks = 32;
 mote_status_t launch_quant_act(const QuantActArgs& a, bool scatter, cudaStream_t stream);
 
 // Router (Eq. 3).  Arguments as mote_route_topk.

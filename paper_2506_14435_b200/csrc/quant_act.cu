@@ -17,8 +17,58 @@
 
 namespace mote {
 
+// Block-wise dispatch of a short call (see dispatch_scan_kernel for the long ones): every CTA of 256 threads scans the
+// router's block counts for itself, one warp per expert, lane = block.  s_pre[e][b]: pairs of expert e in earlier blocks;
+// s_first[e]: first sorted row of expert e.  A kernel of its own for this is 4.4 us of launch, load and store latency
+// (T <= 512); here it is one more trip to L2 behind the router.
+struct InlineScan {
+  uint16_t pre[MOTE_MAX_EXPERTS][kInlineScanBlocks];
+  int count[MOTE_MAX_EXPERTS], first[MOTE_MAX_EXPERTS];
+};
+__device__ __forceinline__ int scan_inclusive(int v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += n;
+  }
+  return v;
+}
+__device__ __forceinline__ void scan_block_counts(const QuantActArgs& a, InlineScan& sc) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, E = a.E;
+  for (int e = warp; e < E; e += 8) {
+    const int v = lane < a.n_blk ? __ldcg(a.blk_hist + e * blk_stride(a.n_blk) + lane) : 0;
+    const int incl = scan_inclusive(v, lane);
+    sc.pre[e][lane] = (uint16_t)(incl - v);
+    if (lane == 31) sc.count[e] = incl;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const int c0 = lane < E ? sc.count[lane] : 0, c1 = lane + 32 < E ? sc.count[lane + 32] : 0;
+    const int n0 = (c0 + 127) / 128, n1 = (c1 + 127) / 128;
+    const int r0 = scan_inclusive(c0, lane), t0 = scan_inclusive(n0, lane);
+    const int r1 = scan_inclusive(c1, lane) + __shfl_sync(0xffffffffu, r0, 31);
+    const int t1 = scan_inclusive(n1, lane) + __shfl_sync(0xffffffffu, t0, 31);
+    sc.first[lane] = r0 - c0; sc.first[lane + 32] = r1 - c1;
+    if (blockIdx.x == 0) {
+      if (lane < E) a.offsets_out[lane] = r0 - c0;
+      if (lane + 32 < E) a.offsets_out[lane + 32] = r1 - c1;
+      for (int i = 0; i < n0; ++i) a.tiles_routed[1 + t0 - n0 + i] = make_int4(lane, r0 - c0 + 128 * i, min(128, c0 - 128 * i), 0);
+      for (int i = 0; i < n1; ++i) a.tiles_routed[1 + t1 - n1 + i] = make_int4(lane + 32, r1 - c1 + 128 * i, min(128, c1 - 128 * i), 0);
+      if (lane == 31) {
+        a.offsets_out[E] = r1;
+        a.tiles_routed[0] = make_int4(t1, 0, 0, 0);
+      }
+      const int T = (int)a.T, n = (T + 127) / 128;
+      for (int i = lane; i < n; i += 32) a.tiles_shared[1 + i] = make_int4(0, i * 128, min(128, T - i * 128), 0);
+      if (lane == 0) a.tiles_shared[0] = make_int4(n, 0, 0, 0);
+    }
+  }
+  __syncthreads();
+}
+
 template <int kUnits, bool kScatter>
 __global__ void __launch_bounds__(256, kUnits <= 2 ? 4 : 0) quant_act_kernel(QuantActArgs a) {
+  __shared__ InlineScan s_scan;
   __shared__ float s_max[8];
   __shared__ int s_sum[8];
   const int G = a.group;                          // threads per row
@@ -99,15 +149,16 @@ __global__ void __launch_bounds__(256, kUnits <= 2 ? 4 : 0) quant_act_kernel(Qua
     for (int i = 0; i < nw; ++i) s += s_sum[w0 + i];
     local_sum = s;
   }
-  if (!row_ok) return;
-
   // everything above depends on x only; the routing of the kernels before this one is needed from here on
   if (kScatter) pdl_wait();
+  const bool scan = kScatter && a.blk_hist != nullptr;
+  if (scan) scan_block_counts(a, s_scan);
+  if (!row_ok) return;
   const int n_dst = kScatter ? a.k : 1;
   for (int j = 0; j < n_dst; ++j) {
     int64_t dst = row;
     if (kScatter) {
-      if (a.blk_base) {
+      if (scan || a.blk_base) {
         // sorted row = first row of (block, expert) + number of earlier pairs of the block with that
         // expert; a row group is made of whole warps, so the ballots below see converged warps
         const int pair = (int)row * a.k + j;
@@ -120,7 +171,7 @@ __global__ void __launch_bounds__(256, kUnits <= 2 ? 4 : 0) quant_act_kernel(Qua
           const bool m = pp < pair && a.topk_idx[pp] == e;
           rank += __popc(__ballot_sync(0xffffffffu, m));
         }
-        dst = a.blk_base[e * blk_stride(a.n_blk) + blk] + rank;
+        dst = (scan ? s_scan.first[e] + s_scan.pre[e][blk] : a.blk_base[e * blk_stride(a.n_blk) + blk]) + rank;
         if (tg == 0) {
           a.perm_out[pair] = (int32_t)dst;
           a.inv_out[dst] = pair;
@@ -393,7 +444,7 @@ mote_status_t launch_quant_act(const QuantActArgs& a, bool scatter, cudaStream_t
   const unsigned blocks = (unsigned)((a.T + rows_per_cta - 1) / rows_per_cta);
 #define MOTE_QA_LAUNCH(U)                                                          \
   do {                                                                             \
-    if (scatter && args.blk_base)                                                   \
+    if (scatter && (args.blk_base || args.blk_hist))                                                   \
       MOTE_CUDA_OK(launch_pdl(quant_act_kernel<U, true>, dim3(blocks), dim3(threads), 0, stream, args)); \
     else if (scatter) quant_act_kernel<U, true><<<blocks, threads, 0, stream>>>(args);  \
     else quant_act_kernel<U, false><<<blocks, threads, 0, stream>>>(args);         \

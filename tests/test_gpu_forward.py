@@ -211,6 +211,18 @@ def test_rtn_shared_expert(mote, d, f, E, k, T, kw, path, bits):
     check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
 
 
+@pytest.mark.parametrize("E,k,T,kw", [
+    (1, 1, 1, {}),
+    (64, 8, 16, {}), (64, 8, 17, {}),                     # one block of the router; a second one of one token
+    (33, 2, 500, dict(bias="zipf")),                      # experts in both halves of the scan's warp, several tiles each
+    (64, 3, 512, dict(bias="normal")), (64, 3, 513, {}),  # the most blocks that every CTA of Q_a(x) scans; one more
+])
+def test_dispatch_of_short_prefills(mote, E, k, T, kw):
+    wl = synth.custom("scan", 128, 128, E, k, T, 6000 + E + T, **kw)
+    master, layer_or, layer_gpu = _setup(mote, wl, TENSOR)
+    check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
+
+
 @pytest.mark.parametrize("bits", [16, 8, 4])
 @pytest.mark.parametrize("d,f,E,k,T,kw", [
     (128, 512, 2, 1, 33, {}),                             # the smallest: one row tile per kind, one pipeline step of gate/up
