@@ -163,8 +163,6 @@ __global__ void __launch_bounds__(kRmWarps * 32, NE <= 2 ? 4 : 0) route_topk_mma
   __shared__ float s_logits[16][NE * 8];
   __shared__ int s_hist[NE * 8];                      // pairs per expert among this CTA's 16 tokens
   if (threadIdx.x < NE * 8) s_hist[threadIdx.x] = 0;
-  // first kernel of a layer call on the tensor path: clears the call's device status word
-  if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int64_t t0 = int64_t(blockIdx.x) * 16;
   const uint16_t* xa = x + min(t0 + g, T - 1) * int64_t(d) + t * 8;       // rows past the end alias the last row
@@ -180,6 +178,14 @@ __global__ void __launch_bounds__(kRmWarps * 32, NE <= 2 ? 4 : 0) route_topk_mma
   const int n_steps = d / 32;
   const int base = n_steps / kRmWarps, rem = n_steps % kRmWarps;
   const int sb = warp * base + min(warp, rem), se = sb + base + (warp < rem ? 1 : 0);
+  // Launched as a programmatic dependent: this much runs under the tail of the kernel ahead, which may write x.  The
+  // router weights are nobody's output; their way from HBM is most of a short call's time here.
+  for (int s = sb; s < se; ++s)
+#pragma unroll
+    for (int n = 0; n < NE; ++n) asm volatile("prefetch.global.L2 [%0];" ::"l"(wrow[n] + s * 32));
+  pdl_wait();
+  // first kernel of a layer call on the tensor path: clears the call's device status word
+  if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0u;
   // token loads in flight per lane; two for E > 8 keep the kernel at 64 registers, i.e. four CTAs per
   // SM, so that the 512 CTAs of an 8192-token prefill are resident at once (router 38 -> 24 us there)
   constexpr int kAhead = (NE >= 2) ? 2 : 4;
@@ -303,10 +309,14 @@ mote_status_t launch_route_topk(const void* x, int64_t T, int d, const float* Wr
   if (d % 32 == 0) {
     const unsigned blocks = (unsigned)((T + 15) / 16);
     const int ne = (E + 7) / 8;
-    if (ne <= 1) route_topk_mma_kernel<1><<<blocks, kRmWarps * 32, 0, stream>>>(xp, T, d, Wr, bias, E, k, norm_topk, idx, w, logits, blk_hist, zero_word);
-    else if (ne <= 2) route_topk_mma_kernel<2><<<blocks, kRmWarps * 32, 0, stream>>>(xp, T, d, Wr, bias, E, k, norm_topk, idx, w, logits, blk_hist, zero_word);
-    else if (ne <= 4) route_topk_mma_kernel<4><<<blocks, kRmWarps * 32, 0, stream>>>(xp, T, d, Wr, bias, E, k, norm_topk, idx, w, logits, blk_hist, zero_word);
-    else route_topk_mma_kernel<8><<<blocks, kRmWarps * 32, 0, stream>>>(xp, T, d, Wr, bias, E, k, norm_topk, idx, w, logits, blk_hist, zero_word);
+#define MOTE_ROUTE_LAUNCH(NE_)                                                                                     \
+  MOTE_CUDA_OK(launch_pdl(route_topk_mma_kernel<NE_>, dim3(blocks), dim3(kRmWarps * 32), 0, stream, xp, T, d, Wr, bias, E, k, \
+                          norm_topk, idx, w, logits, blk_hist, zero_word))
+    if (ne <= 1) MOTE_ROUTE_LAUNCH(1);
+    else if (ne <= 2) MOTE_ROUTE_LAUNCH(2);
+    else if (ne <= 4) MOTE_ROUTE_LAUNCH(4);
+    else MOTE_ROUTE_LAUNCH(8);
+#undef MOTE_ROUTE_LAUNCH
   } else {
     const int per_cta = kRouteWarps * kRouteTok;
     const unsigned blocks = (unsigned)((T + per_cta - 1) / per_cta);
