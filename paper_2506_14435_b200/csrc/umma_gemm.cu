@@ -868,17 +868,18 @@ struct GemmSetup {
 static bool setup_ternary(GemmSetup& u, const TernaryGemmArgs& g, bool gateup, const int4* tiles, int max_mtiles,
                           const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status) {
   int bn = gateup ? 256 : pick_bn(g.N);
-  // a down projection with few row tiles: 128-wide tiles double the items (the weights are the
-  // traffic here, and they are read once either way)
-  if (!gateup && bn > 128) {
+  // a down projection with few row tiles: the narrowest tiles (at least 64 wide) that are no more than the SMs (the
+  // weights are the traffic here, and they are read once either way)
+  if (!gateup) {
     const int sms = device_sm_count();
-    if (max_mtiles * (g.N / bn) * 2 <= sms) bn = 128;
+    for (int n = 64; n < bn; n += 32)
+      if (g.N % n == 0 && max_mtiles * (g.N / n) <= sms) bn = n;
   }
   // second weight map: the up matrix (gate/up), or the rows beyond 128 of a down tile
   if (!make_map_2d(&u.ta, g.qa, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.P, (uint64_t)g.K, 128, 128,
                    CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_map_2d(&u.tb0, g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N, (uint64_t)g.K / 4, 128, 32,
-                   CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !make_map_2d(&u.tb0, g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N, (uint64_t)g.K / 4,
+                   std::min(bn, 128), 32, CU_TENSOR_MAP_SWIZZLE_NONE) ||
       !make_map_2d(&u.tb1, gateup ? g.w1 : g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N,
                    (uint64_t)g.K / 4, (gateup || bn <= 128) ? 128 : bn - 128, 32, CU_TENSOR_MAP_SWIZZLE_NONE))
     return false;

@@ -230,6 +230,8 @@ def test_dispatch_of_short_prefills(mote, E, k, T, kw):
     (256, 4864, 16, 2, 64, dict(outlier_frac=0.01)),      # sixteen K splits, odd numbers of pipeline steps per split
     (1536, 384, 8, 2, 333, dict(norm_topk=0)),            # more items than SMs: CTAs walk from one kind to the other
     (2048, 512, 8, 1, 1000, {}),                          # the most row tiles: two K splits
+    (384, 256, 3, 1, 48, {}), (640, 256, 3, 1, 48, {}),   # routed down tiles of 64 rows; 640 is not a multiple of 96
+    (1536, 256, 8, 2, 64, {}),                            # ... of 96 rows
 ])
 def test_short_prefill_pairs_of_gemms(mote, d, f, E, k, T, kw, bits):
     wl = synth.custom("pair", d, f, E, k, T, 5000 + d + f + T, **kw)
