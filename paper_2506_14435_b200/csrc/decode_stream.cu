@@ -704,11 +704,13 @@ __device__ __forceinline__ void gateup_shared_tile(const DecodeGateUpArgs& a, in
 // code expansion of the RTN widths costs the bf16 kernel no registers
 // The bf16 kernel for 9..16 tokens is held to 72 registers (it takes 80 left alone): seven CTAs per SM
 // instead of six, 8 % off the gate/up stream at T = 16.  (96 registers for 17..32 tokens: no gain.)
+// The kernels for 17..32 tokens are held to 128 registers, four CTAs per SM (the bf16 one takes that many left alone; the
+// 4-bit one came out at more: 291 -> 275 us per three layers of 2048 x 11008, 4 experts, 32 tokens).
 // The other instantiations must stay without a minimum (0): a minimum of one CTA is not the same
 // to the compiler as none (it then plans for all 512 registers a thread could have, and the
 // streams of 1..8 and 17..32 tokens came out 9-50 % slower).
 template <int NTB, int kShBits>
-__global__ void __launch_bounds__(kGuWarps * 32, (NTB == 2 && kShBits == 16) ? 7 : 0) decode_gateup_kernel(DecodeGateUpArgs a) {
+__global__ void __launch_bounds__(kGuWarps * 32, (NTB == 2 && kShBits == 16) ? 7 : NTB == 4 ? 4 : 0) decode_gateup_kernel(DecodeGateUpArgs a) {
   __shared__ ExpertList s_list;
   __shared__ float s_part[kGuWarps * NTB * 4 * 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -746,7 +748,7 @@ __global__ void __launch_bounds__(kGuWarps * 32, (NTB == 2 && kShBits == 16) ? 7
 }
 
 // ------------------------------------------------------------------------------------------------
-// decode_down: kDownWarps warps per CTA split the reduction dimension f of one 16-row tile of d.
+// decode_down: the warps of a CTA (kDownWarps) split the reduction dimension f of one 16-row tile of d.
 // ------------------------------------------------------------------------------------------------
 struct DecodeDownArgs {
   DecodeCommon c;
@@ -768,9 +770,8 @@ struct DecodeDownArgs {
   uint32_t* tile_count;         // [d/16] zero on entry
 };
 
-constexpr int kDownWarps = 16;
 
-template <int NT>
+template <int NT, int kDownWarps>
 __device__ __forceinline__ void down_routed_tile(const DecodeDownArgs& a, int e, int tile, int warp, int lane,
                                                  int* s_part) {
   const int d = a.c.d, f = a.c.f;
@@ -825,7 +826,7 @@ __device__ __forceinline__ void down_routed_tile(const DecodeDownArgs& a, int e,
   __syncthreads();
 }
 
-template <int NT, int kShBits>
+template <int NT, int kShBits, int kDownWarps>
 __device__ __forceinline__ void down_shared_tile(const DecodeDownArgs& a, int tile, int warp, int lane, float* s_part) {
   const int d = a.c.d, f = a.c.f, T = a.c.T;
   const int g = lane >> 2, t = lane & 3;
@@ -871,9 +872,8 @@ __device__ __forceinline__ void down_shared_tile(const DecodeDownArgs& a, int ti
 // its stores of the item; the count is kept per tile, so the combines of different tiles run in
 // parallel on whichever CTAs arrive last.
 __device__ __forceinline__ void down_tile_done(const DecodeDownArgs& a, int tile, int n_producers, int* s_last) {
-  __threadfence();                                   // this thread's y / s values are visible device-wide
-  __syncthreads();
   if (threadIdx.x == 0) {
+    __threadfence();                                 // with the barrier ahead: the CTA's y / s values are visible device-wide
     const uint32_t old = atomicAdd(a.tile_count + tile, 1u);
     *s_last = (old == (uint32_t)n_producers - 1u);
     if (*s_last) a.tile_count[tile] = 0u;            // left clean for the next call
@@ -897,9 +897,13 @@ __device__ __forceinline__ void down_tile_done(const DecodeDownArgs& a, int tile
 // one CTA per SM and was 8-15 % slower; every one-tile kernel is capped too: left alone the bf16 one
 // takes 106 registers, one CTA per SM, and the step is 5-10 % slower.  The 16-token 4-bit expansion
 // would spill too much under that cap.)
-template <int NTB, int kShBits>
+// 17 to 32 tokens at 128 registers: CTAs of eight warps, two per SM, so that one streams while the other adds up, where
+// there are more than two items per SM (2048 x 11008, 16 experts, 32 tokens: kernel 86 -> 74 us; four warps: the same);
+// CTAs of sixteen below that (896 x 4864, 4 experts, 17 tokens: layer 35.0 against 36.1 us).  Up to 16 tokens eight warps
+// are slower (382 -> 460 us per eight layers of one token: a shared tile's 352 KB come in too slowly).
+template <int NTB, int kShBits, int kDownWarps>
 __global__ void __launch_bounds__(kDownWarps * 32,
-                                  (NTB == 1 || (NTB == 2 && kShBits != 4)) ? 2 : 1)
+                                  (NTB == 1 || (NTB == 2 && kShBits != 4)) ? 2 : 16 / kDownWarps)
 decode_down_kernel(DecodeDownArgs a) {
   __shared__ ExpertList s_list;
   __shared__ int s_last;
@@ -921,17 +925,17 @@ decode_down_kernel(DecodeDownArgs a) {
       waited = true;
     }
     if (item < n_shared) {
-      down_shared_tile<NTB, kShBits>(a, item, warp, lane, s_part);
+      down_shared_tile<NTB, kShBits, kDownWarps>(a, item, warp, lane, s_part);
       down_tile_done(a, item, 1 + s_list.n, &s_last);
     } else {
       const int r = item - n_shared;
       const int e = s_list.id[r / tiles];
       const int tile = r % tiles;
       const int nt = (a.c.offsets[e + 1] - a.c.offsets[e] + 7) / 8;
-      if (NTB == 1 || nt <= 1) down_routed_tile<1>(a, e, tile, warp, lane, ip);
-      else if (NTB == 2 || nt <= 2) down_routed_tile<(NTB >= 2 ? 2 : 1)>(a, e, tile, warp, lane, ip);
-      else if (NTB == 4 || nt <= 4) down_routed_tile<(NTB >= 4 ? 4 : 1)>(a, e, tile, warp, lane, ip);
-      else down_routed_tile<(NTB >= 8 ? 8 : 1)>(a, e, tile, warp, lane, ip);
+      if (NTB == 1 || nt <= 1) down_routed_tile<1, kDownWarps>(a, e, tile, warp, lane, ip);
+      else if (NTB == 2 || nt <= 2) down_routed_tile<(NTB >= 2 ? 2 : 1), kDownWarps>(a, e, tile, warp, lane, ip);
+      else if (NTB == 4 || nt <= 4) down_routed_tile<(NTB >= 4 ? 4 : 1), kDownWarps>(a, e, tile, warp, lane, ip);
+      else down_routed_tile<(NTB >= 8 ? 8 : 1), kDownWarps>(a, e, tile, warp, lane, ip);
       down_tile_done(a, tile, 1 + s_list.n, &s_last);
     }
   }
@@ -980,7 +984,11 @@ mote_status_t launch_decode_stream(const DecodeStreamArgs& p, int phase, cudaStr
     ga.hs = static_cast<uint16_t*>(p.hs); ga.tap_gate = p.tap_gate; ga.tap_up = p.tap_up;
     const int tiles = f / 8, quads = (tiles + kGuWarps - 1) / kGuWarps;
     const int max_items = tiles + std::min<int>(E, T * k) * quads;
-    const int grid = std::min(max_items, sms * 12);
+    // as many CTAs as are resident at once: each walks over its items, and the start of a CTA (list of experts, first
+    // loads) is paid once.  With twelve per SM in several waves: eight layers of 2048 x 11008 at 32 tokens 1326 against
+    // 1288 us, at one token 383 against 378; three layers at 9 tokens 353 against 330.  (33 and more tokens: not measured
+    // to gain, few CTAs fit.)
+    const int grid = std::min(max_items, sms * (ntb == 4 ? 4 : ntb == 8 ? 12 : 7));
 #define MOTE_GU_LAUNCH(NTB_, BITS_) \
   MOTE_CUDA_OK(launch_pdl(decode_gateup_kernel<NTB_, BITS_>, dim3(grid), dim3(kGuWarps * 32), 0, stream, ga))
 #define MOTE_GU_BITS(NTB_)                                 \
@@ -1008,24 +1016,26 @@ mote_status_t launch_decode_stream(const DecodeStreamArgs& p, int phase, cudaStr
   da.hs = static_cast<const uint16_t*>(p.hs); da.y = p.y; da.s = p.s; da.tap_down = p.tap_down;
   const int tiles = d / 16;
   const int max_items = tiles + std::min<int>(E, T * k) * tiles;
-  const int grid = std::min(max_items, sms * 3);
-  const size_t smem = size_t(kDownWarps) * ntb * 4 * 32 * sizeof(float);
+  const int warps = ntb == 4 && max_items > 2 * sms ? 8 : 16;
+  const int grid = std::min(max_items, sms * (48 / warps));
+  const size_t smem = size_t(warps) * ntb * 4 * 32 * sizeof(float);
   static PerDeviceOnce down_attr16, down_attr8, down_attr4;
-  MOTE_CUDA_OK(set_max_dynamic_smem(down_attr16, decode_down_kernel<8, 16>, 65536));
-  MOTE_CUDA_OK(set_max_dynamic_smem(down_attr8, decode_down_kernel<8, 8>, 65536));
-  MOTE_CUDA_OK(set_max_dynamic_smem(down_attr4, decode_down_kernel<8, 4>, 65536));
-#define MOTE_DN_LAUNCH(NTB_, BITS_) \
-  MOTE_CUDA_OK(launch_pdl(decode_down_kernel<NTB_, BITS_>, dim3(grid), dim3(kDownWarps * 32), smem, stream, da))
-#define MOTE_DN_BITS(NTB_)                                 \
-  do {                                                     \
-    if (p.shared_bits == 8) MOTE_DN_LAUNCH(NTB_, 8);       \
-    else if (p.shared_bits == 4) MOTE_DN_LAUNCH(NTB_, 4);  \
-    else MOTE_DN_LAUNCH(NTB_, 16);                         \
+  MOTE_CUDA_OK(set_max_dynamic_smem(down_attr16, decode_down_kernel<8, 16, 16>, 65536));
+  MOTE_CUDA_OK(set_max_dynamic_smem(down_attr8, decode_down_kernel<8, 8, 16>, 65536));
+  MOTE_CUDA_OK(set_max_dynamic_smem(down_attr4, decode_down_kernel<8, 4, 16>, 65536));
+#define MOTE_DN_LAUNCH(NTB_, BITS_, W_) \
+  MOTE_CUDA_OK(launch_pdl(decode_down_kernel<NTB_, BITS_, W_>, dim3(grid), dim3(warps * 32), smem, stream, da))
+#define MOTE_DN_BITS(NTB_, W_)                                 \
+  do {                                                         \
+    if (p.shared_bits == 8) MOTE_DN_LAUNCH(NTB_, 8, W_);       \
+    else if (p.shared_bits == 4) MOTE_DN_LAUNCH(NTB_, 4, W_);  \
+    else MOTE_DN_LAUNCH(NTB_, 16, W_);                         \
   } while (0)
-  if (ntb == 1) MOTE_DN_BITS(1);
-  else if (ntb == 2) MOTE_DN_BITS(2);
-  else if (ntb == 4) MOTE_DN_BITS(4);
-  else MOTE_DN_BITS(8);
+  if (ntb == 1) MOTE_DN_BITS(1, 16);
+  else if (ntb == 2) MOTE_DN_BITS(2, 16);
+  else if (ntb == 4 && warps == 8) MOTE_DN_BITS(4, 8);
+  else if (ntb == 4) MOTE_DN_BITS(4, 16);
+  else MOTE_DN_BITS(8, 16);
 #undef MOTE_DN_BITS
 #undef MOTE_DN_LAUNCH
   ++g_launch_count;

@@ -211,6 +211,21 @@ def test_rtn_shared_expert(mote, d, f, E, k, T, kw, path, bits):
     check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
 
 
+@pytest.mark.parametrize("bits", [16, 8, 4])
+@pytest.mark.parametrize("d,f,E,k,T,kw", [
+    (256, 512, 4, 1, 20, {}),                             # few down items: sixteen warps each
+    (1024, 256, 8, 2, 17, {}),                            # many: eight warps, one reduction step among them
+    (1088, 4864, 8, 2, 32, dict(bias="zipf")),            # ... and 19 uneven steps, experts of one to four token tiles
+])
+def test_stream_path_17_to_32_tokens(mote, d, f, E, k, T, kw, bits):
+    wl = synth.custom("mid", d, f, E, k, T, 7000 + d + T, **kw)
+    master, layer_or, layer_gpu = _setup(mote, wl, STREAM)
+    if bits != 16:
+        layer_or = O.quantize_shared(layer_or, bits)
+        layer_gpu = layer_gpu.quantize_shared(bits)
+    check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
+
+
 @pytest.mark.parametrize("E,k,T,kw", [
     (1, 1, 1, {}),
     (64, 8, 16, {}), (64, 8, 17, {}),                     # one block of the router; a second one of one token
