@@ -1,6 +1,6 @@
 // Absmean ternary weight quantizer with INT2 packing (Eq. 7, 9, 10; storage per Section 3.1).
 //
-// Two launches per matrix (after a clear of the bins), both bound by HBM; 83 -> 43 us per 11008 x 2048
+// Two launches per matrix (after a clear of the bins), both bound by HBM; 83 -> 38 us per 11008 x 2048
 // fp32 matrix against three launches with a branch per element and a division per code:
 //   1. abs_sum_alpha   exact accumulation of sum |w|: each fp32 magnitude is split into its
 //                      24-bit integer significand and its exponent; significands are added (shifted
@@ -84,7 +84,7 @@ __device__ __forceinline__ void abs_acc_flush_warp(AbsAcc& st, unsigned long lon
 }
 
 // Sixteen elements at once (called by whole warps).  Where all of them lie in the window (32 binades,
-// placed 24 below the largest of the warp's first weights) they need one range check together and eight instructions
+// placed 24 below the largest of the warp's first weights) they need one range check together and six instructions
 // each: the magnitude less the window's lower edge, in one add (bits + bits drops the sign), is at once
 // the shift (top byte) and, compared unsigned, the check.  Zeros and outliers go one by one.
 __device__ __forceinline__ void abs_acc_add16(AbsAcc& st, const uint32_t (&bits)[16], unsigned long long* sbins) {
@@ -104,7 +104,8 @@ __device__ __forceinline__ void abs_acc_add16(AbsAcc& st, const uint32_t (&bits)
     const uint32_t x = bits[j] + bits[j] + edge, sh = x >> 24;
     const uint32_t mant = (bits[j] & 0x7FFFFFu) | 0x800000u;
     top = max(top, x);
-    sum += ((unsigned long long)__funnelshift_l(mant, 0u, sh) << 32) | __funnelshift_l(0u, mant, sh);
+    sum += (unsigned long long)mant * (1u << (sh & 31u));            // the shift as a wide multiply-add: one instruction of
+                                                                     // the FMA pipe for four of the busier integer ALU
   }
   if (st.base > 0 && top < (32u << 24)) {
     st.acc += sum;
@@ -142,12 +143,18 @@ constexpr int kLimbs = 12;
 __device__ __forceinline__ void finalize_alpha(const unsigned long long* s_bins, unsigned long long* s_limb, double count,
                                                float* __restrict__ alpha) {
   const int lane = threadIdx.x & 31;
+  // only bins that hold something (a handful: the weights' binades over 32): going over all of them, three limbs each,
+  // took the one warp 7 us
   unsigned long long col = 0ull;                           // at most 3 x 32 parts below 2^32
-  for (int e = max(32 * (lane - 2), 0); e < min(32 * (lane + 1) + 1, 255); ++e) {
-    const int sft = (e ? e : 1) - 1, part = lane - (sft >> 5);
-    if (part < 0 || part > 2) continue;
-    const unsigned __int128 sv = (unsigned __int128)s_bins[e] << (sft & 31);   // < 2^95
-    col += (uint32_t)(sv >> (32 * part));
+  for (int e0 = 0; e0 < 255; e0 += 32) {
+    uint32_t used = __ballot_sync(0xffffffffu, e0 + lane < 255 && s_bins[min(e0 + lane, 254)] != 0ull);
+    while (used) {
+      const int e = e0 + __ffs(used) - 1, sft = (e ? e : 1) - 1, part = lane - (sft >> 5);
+      used &= used - 1u;
+      if (part < 0 || part > 2) continue;
+      const unsigned __int128 sv = (unsigned __int128)s_bins[e] << (sft & 31);   // < 2^95
+      col += (uint32_t)(sv >> (32 * part));
+    }
   }
   if (lane < kLimbs) s_limb[lane] = col;
   __syncwarp();
