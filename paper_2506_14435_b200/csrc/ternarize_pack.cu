@@ -188,8 +188,11 @@ __device__ __forceinline__ void finalize_alpha(const unsigned long long* s_bins,
 
 // One warp takes items of 512 elements; the next item is on its way while one is added.  The last bin
 // (never counted into) is the grid's arrival counter.
+// One CTA of 1024 threads per SM: a quarter of the CTAs meet at the bins' atomics that four of 256 would send there (three
+// matrices of 2048 x 11008: fp32 117 -> 114 us, bf16 102.7 -> 100).
+constexpr int kSumThreads = 1024;
 template <bool kBf16>
-__global__ void __launch_bounds__(256, 4) abs_sum_alpha_kernel(const void* __restrict__ W, int64_t total, double count,
+__global__ void __launch_bounds__(kSumThreads, 1) abs_sum_alpha_kernel(const void* __restrict__ W, int64_t total, double count,
                                                             unsigned long long* __restrict__ bins, float* __restrict__ alpha) {
   __shared__ unsigned long long sbins[kBins];
   __shared__ unsigned long long s_limb[kLimbs];
@@ -272,11 +275,11 @@ static mote_status_t ternarize_with_bins(const void* W, int w_dtype, int64_t tot
   MOTE_CUDA_OK(cudaMemsetAsync(bins, 0, kBins * sizeof(unsigned long long), stream));
   const int threads = 256;
   const int64_t ctas = (total + 512 * 8 - 1) / (512 * 8);            // 512 elements per warp
-  const int blocks_a = (int)std::min<int64_t>(ctas, int64_t(device_sm_count()) * 4);
+  const int blocks_a = (int)std::min<int64_t>((ctas + 3) / 4, int64_t(device_sm_count()));
   const int blocks_c = (int)std::min<int64_t>(ctas, int64_t(device_sm_count()) * 16);
   const bool bf16 = w_dtype == MOTE_DTYPE_BF16;
-  if (bf16) abs_sum_alpha_kernel<true><<<blocks_a, threads, 0, stream>>>(W, total, (double)total, bins, alpha);
-  else abs_sum_alpha_kernel<false><<<blocks_a, threads, 0, stream>>>(W, total, (double)total, bins, alpha);
+  if (bf16) abs_sum_alpha_kernel<true><<<blocks_a, kSumThreads, 0, stream>>>(W, total, (double)total, bins, alpha);
+  else abs_sum_alpha_kernel<false><<<blocks_a, kSumThreads, 0, stream>>>(W, total, (double)total, bins, alpha);
   MOTE_LAUNCH_OK();
   if (bf16) MOTE_CUDA_OK(launch_pdl(pack_codes_kernel<true>, dim3(blocks_c), dim3(threads), 0, stream, W, total, alpha, packed));
   else MOTE_CUDA_OK(launch_pdl(pack_codes_kernel<false>, dim3(blocks_c), dim3(threads), 0, stream, W, total, alpha, packed));
