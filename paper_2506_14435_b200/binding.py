@@ -29,6 +29,9 @@ class mote_layer_t(C.Structure):
                 ("sh_gate_scale", C.c_void_p), ("sh_up_scale", C.c_void_p), ("sh_down_scale", C.c_void_p)]
 
 
+_LAYER_POINTERS = [n for n, t in mote_layer_t._fields_ if t is C.c_void_p]   # 11 ahead of shared_bits, 3 behind
+
+
 TAP_FIELDS = ["topk_idx", "topk_w", "offsets", "perm", "qx", "beta_x", "acc_gate", "acc_up", "h_bf16",
               "qh", "beta_h", "acc_down", "y", "shared_out"]
 
@@ -105,7 +108,8 @@ def _ptr(t):
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the handle alone: building the Stream object takes about as long as launching a kernel
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _need_cuda(*ts):
@@ -270,15 +274,12 @@ class MoteLayer:
 
     def struct(self) -> mote_layer_t:
         t = self.tensors
-        s = mote_layer_t(self.d, self.f, self.E, self.k, self.norm_topk, self.path)
-        for name in ("Wr", "router_bias", "gate_packed", "up_packed", "down_packed", "alpha_gate", "alpha_up",
-                     "alpha_down", "sh_gate", "sh_up", "sh_down", "sh_gate_scale", "sh_up_scale", "sh_down_scale"):
-            setattr(s, name, None if t[name] is None else t[name].data_ptr())
-        s.shared_bits = self.shared_bits
-        return s
+        p = [None if t[n] is None else t[n].data_ptr() for n in _LAYER_POINTERS]
+        return mote_layer_t(self.d, self.f, self.E, self.k, self.norm_topk, self.path, *p[:11], self.shared_bits, *p[11:])
 
-    def workspace(self, T: int, host_staging: bool = False) -> torch.Tensor:
-        need = lib.mote_layer_workspace_bytes(C.byref(self.struct()), T)
+    def workspace(self, T: int, host_staging: bool = False, struct: mote_layer_t | None = None) -> torch.Tensor:
+        """struct: self.struct(), from a caller that has one at hand."""
+        need = lib.mote_layer_workspace_bytes(C.byref(self.struct() if struct is None else struct), T)
         if need == 0:
             raise MoteError(2, "mote_layer_workspace_bytes")
         if host_staging:
@@ -305,8 +306,8 @@ def mote_moe_forward(layer: MoteLayer, x: torch.Tensor, residual=None, out=None,
     T = x.shape[0]
     if out is None:
         out = torch.empty_like(x)
-    ws = layer.workspace(T)
     s = layer.struct()
+    ws = layer.workspace(T, struct=s)
     tp = None
     if taps is not None:
         tp = mote_taps_t()
@@ -321,8 +322,8 @@ def mote_moe_forward(layer: MoteLayer, x: torch.Tensor, residual=None, out=None,
 def mote_moe_forward_host(layer: MoteLayer, x_host: torch.Tensor, out_host: torch.Tensor, residual_host=None):
     """Same layer with (pinned) host tensors in and out; synchronises the stream."""
     T = x_host.shape[0]
-    ws = layer.workspace(T, host_staging=True)
     s = layer.struct()
+    ws = layer.workspace(T, host_staging=True, struct=s)
     _check(lib.mote_moe_forward_host(C.byref(s), _ptr(x_host), _ptr(residual_host), T, _ptr(out_host), _ptr(ws),
                                      ws.numel(), _stream()), "mote_moe_forward_host")
     return out_host
