@@ -986,9 +986,11 @@ mote_status_t launch_decode_stream(const DecodeStreamArgs& p, int phase, cudaStr
     const int max_items = tiles + std::min<int>(E, T * k) * quads;
     // as many CTAs as are resident at once: each walks over its items, and the start of a CTA (list of experts, first
     // loads) is paid once.  With twelve per SM in several waves: eight layers of 2048 x 11008 at 32 tokens 1326 against
-    // 1288 us, at one token 383 against 378; three layers at 9 tokens 353 against 330.  (33 and more tokens: not measured
-    // to gain, few CTAs fit.)
-    const int grid = std::min(max_items, sms * (ntb == 4 ? 4 : ntb == 8 ? 12 : 7));
+    // 1288 us, at one token 382.5 against 378; three layers at 9 tokens 353 against 330.  Up to 8 tokens with more than
+    // two items per resident CTA the waves stay: their order evens out unequal items (1536 x 8960, 8 experts, 8 tokens:
+    // 52.7 against 54.6 us).  (33 and more tokens: few CTAs fit, not measured to gain.)
+    const int per_sm = ntb == 4 ? 4 : ntb == 2 || (ntb == 1 && max_items <= 14 * sms) ? 7 : 12;
+    const int grid = std::min(max_items, sms * per_sm);
 #define MOTE_GU_LAUNCH(NTB_, BITS_) \
   MOTE_CUDA_OK(launch_pdl(decode_gateup_kernel<NTB_, BITS_>, dim3(grid), dim3(kGuWarps * 32), 0, stream, ga))
 #define MOTE_GU_BITS(NTB_)                                 \
