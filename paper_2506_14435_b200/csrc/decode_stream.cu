@@ -826,6 +826,10 @@ __device__ __forceinline__ void down_routed_tile(const DecodeDownArgs& a, int e,
   __syncthreads();
 }
 
+// A tile's sum over f is made of kDownSlices partial sums added in order, whatever the CTA's number of warps: which
+// CTA size a call gets (it depends on d, E and k) must not show in its result.
+constexpr int kDownSlices = 16;
+
 template <int NT, int kShBits, int kDownWarps>
 __device__ __forceinline__ void down_shared_tile(const DecodeDownArgs& a, int tile, int warp, int lane, float* s_part) {
   const int d = a.c.d, f = a.c.f, T = a.c.T;
@@ -834,14 +838,22 @@ __device__ __forceinline__ void down_shared_tile(const DecodeDownArgs& a, int ti
   const uint16_t* tok[NT];
 #pragma unroll
   for (int n = 0; n < NT; ++n) tok[n] = (n * 8 + g) < T ? a.hs + int64_t(n * 8 + g) * f : nullptr;
-  float acc[NT][4];
+  auto add_up = [&](int slice) {
+    float acc[NT][4];
 #pragma unroll
-  for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.0f;
-  shared_rows<NT, kShBits>(a.sh_down.w, drow, drow + 8, f, tok, kDownWarps, warp, lane, acc);
+    for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.0f;
+    shared_rows<NT, kShBits>(a.sh_down.w, drow, drow + 8, f, tok, kDownSlices, slice, lane, acc);
 #pragma unroll
-  for (int n = 0; n < NT; ++n)
+    for (int n = 0; n < NT; ++n)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) s_part[(warp * NT * 4 + n * 4 + i) * 32 + lane] = acc[n][i];
+      for (int i = 0; i < 4; ++i) s_part[(slice * NT * 4 + n * 4 + i) * 32 + lane] = acc[n][i];
+  };
+  if constexpr (kDownWarps == kDownSlices) {
+    add_up(warp);
+  } else {
+#pragma unroll 1
+    for (int slice = warp; slice < kDownSlices; slice += kDownWarps) add_up(slice);
+  }
   __syncthreads();
   const float sc_lo = kShBits == 16 ? 1.0f : a.sh_down.scale[drow];
   const float sc_hi = kShBits == 16 ? 1.0f : a.sh_down.scale[drow + 8];
@@ -851,7 +863,7 @@ __device__ __forceinline__ void down_shared_tile(const DecodeDownArgs& a, int ti
     for (int i = 0; i < 4; ++i) {
       float s = s_part[(n * 4 + i) * 32 + lane];
 #pragma unroll
-      for (int w = 1; w < kDownWarps; ++w) s += s_part[(w * NT * 4 + n * 4 + i) * 32 + lane];
+      for (int w = 1; w < kDownSlices; ++w) s += s_part[(w * NT * 4 + n * 4 + i) * 32 + lane];
       v[i] = s;
     }
 #pragma unroll
@@ -907,7 +919,7 @@ __global__ void __launch_bounds__(kDownWarps * 32,
 decode_down_kernel(DecodeDownArgs a) {
   __shared__ ExpertList s_list;
   __shared__ int s_last;
-  extern __shared__ float s_part[];                       // kDownWarps * NTB * 4 * 32 floats
+  extern __shared__ float s_part[];                       // kDownSlices * NTB * 4 * 32 floats
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // This kernel is let in as soon as Q_a(h) has STARTED (which is after the gate/up kernel and
   // the prologue have completed): the dispatch tables and h_shared are there, and the shared
@@ -1020,7 +1032,7 @@ mote_status_t launch_decode_stream(const DecodeStreamArgs& p, int phase, cudaStr
   const int max_items = tiles + std::min<int>(E, T * k) * tiles;
   const int warps = ntb == 4 && max_items > 2 * sms ? 8 : 16;
   const int grid = std::min(max_items, sms * (48 / warps));
-  const size_t smem = size_t(warps) * ntb * 4 * 32 * sizeof(float);
+  const size_t smem = size_t(kDownSlices) * ntb * 4 * 32 * sizeof(float);
   static PerDeviceOnce down_attr16, down_attr8, down_attr4;
   MOTE_CUDA_OK(set_max_dynamic_smem(down_attr16, decode_down_kernel<8, 16, 16>, 65536));
   MOTE_CUDA_OK(set_max_dynamic_smem(down_attr8, decode_down_kernel<8, 8, 16>, 65536));

@@ -226,6 +226,26 @@ def test_stream_path_17_to_32_tokens(mote, d, f, E, k, T, kw, bits):
     check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
 
 
+@pytest.mark.parametrize("bits", [16, 8, 4])
+@pytest.mark.parametrize("f,T", [(128, 17), (1216, 24), (4864, 32)])      # fewer steps than slices; uneven; several per slice
+def test_shared_expert_does_not_depend_on_the_routed_ones(mote, f, T, bits):
+    # one expert or sixteen beside it decides how many warps a CTA of the down kernel has, not how its sums are grouped
+    wl = synth.custom("slices", 2048, f, 16, 2, T, 7700 + f)
+    many = mote.MoteLayer.from_master(synth.master_layer(wl), path=STREAM)
+    if bits != 16:
+        many = many.quantize_shared(bits)
+    t = {n: v[:1].contiguous() if n == "Wr" or n.endswith("_packed") or n.startswith("alpha_") else v
+         for n, v in many.tensors.items()}
+    one = mote.MoteLayer(2048, f, 1, 1, 1, path=STREAM, shared_bits=bits, **t)
+    x = bf16_tensor(synth.tokens(wl))
+    got = []
+    for layer in (many, one):
+        taps = layer.alloc_taps(T, ["shared_out"])
+        mote.mote_moe_forward(layer, x, taps=taps)
+        got.append(taps["shared_out"])
+    assert torch.equal(*got)
+
+
 @pytest.mark.parametrize("E,k,T,kw", [
     (1, 1, 1, {}),
     (64, 8, 16, {}), (64, 8, 17, {}),                     # one block of the router; a second one of one token
