@@ -8,16 +8,23 @@
 
 namespace mote {
 
-// Its calls are short (a few hundred tokens; long prefills combine in the shared down GEMM's epilogue), so it is bound by
-// the latency of its loads and by how many are in flight: a thread owns four columns, not eight (twice the CTAs), and
-// asks for the partial sums eight at a time and for the expert rows ahead of them.
+// Short prefills (many partial sums of few rows) are bound by the latency of the loads and by how many are in flight: a
+// thread owns four columns (twice the CTAs of eight) and asks for kBatch partial sums at a time and for two expert rows
+// ahead of them.  The CUDA-core path (one sum, any number of rows) and the longer of the short prefills (two to four) are
+// bound by HBM and need the warps instead, so kBatch is no larger than the number of sums: 40, 56, 76 and 99 registers.
+// One kernel of eight for all (99 registers, two CTAs per SM): 44 -> 107 us for 8192 x 2048, one sum, k = 2; with kBatch 1: 46.
+// Two sums of 1024 rows at 2048 x 5632, 16 experts (the whole layer): 219 us with batches of eight, 211 with this.
 __device__ __forceinline__ void add4(float (&acc)[4], const float4& a) { acc[0] += a.x; acc[1] += a.y; acc[2] += a.z; acc[3] += a.w; }
+__device__ __forceinline__ void fma4(float (&acc)[4], float w, const float4& a) {
+  acc[0] = fmaf(w, a.x, acc[0]); acc[1] = fmaf(w, a.y, acc[1]); acc[2] = fmaf(w, a.z, acc[2]); acc[3] = fmaf(w, a.w, acc[3]);
+}
 
+template <int kBatch>
 __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ s, const float* __restrict__ y,
                                                       const float* __restrict__ w, const int32_t* __restrict__ perm,
                                                       const uint16_t* residual, int64_t T, int d, int k,
                                                       uint16_t* out, int n_partials) {
-  constexpr int kBatch = 8, kEarly = 2;
+  constexpr int kEarly = 2;
   const int vec_per_row = d / 4;
   const int64_t total = T * vec_per_row;
   pdl_wait();                            // no-op unless launched as a programmatic dependent
@@ -35,6 +42,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
       }
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     const float* sp = s + t * d + v * 4;
+#pragma unroll 1
     for (int p0 = 0; p0 < n_partials; p0 += kBatch) {   // partial sums of a K-split projection, in order
       float4 sv[kBatch];
 #pragma unroll
@@ -46,19 +54,10 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
         else if (p0 + p < n_partials) add4(acc, sv[p]);
       }
     }
-    for (int j = 0; j < k; ++j) {
-      float wv;
-      float4 a;
-      if (j < kEarly) {
-        wv = j == 0 ? wj[0] : wj[1];
-        a = j == 0 ? yj[0] : yj[1];
-      } else {
-        wv = w[t * k + j];
-        a = *reinterpret_cast<const float4*>(y + int64_t(perm[t * k + j]) * d + v * 4);
-      }
-      acc[0] = fmaf(wv, a.x, acc[0]); acc[1] = fmaf(wv, a.y, acc[1]);
-      acc[2] = fmaf(wv, a.z, acc[2]); acc[3] = fmaf(wv, a.w, acc[3]);
-    }
+#pragma unroll
+    for (int j = 0; j < kEarly; ++j)
+      if (j < k) fma4(acc, wj[j], yj[j]);
+    for (int j = kEarly; j < k; ++j) fma4(acc, w[t * k + j], *reinterpret_cast<const float4*>(y + int64_t(perm[t * k + j]) * d + v * 4));
     if (residual) {
       const uint2 r = *reinterpret_cast<const uint2*>(residual + t * d + v * 4);
       acc[0] += bf16_lo(r.x); acc[1] += bf16_hi(r.x); acc[2] += bf16_lo(r.y); acc[3] += bf16_hi(r.y);
@@ -74,13 +73,21 @@ mote_status_t launch_combine(const float* s, const float* y, const float* w, con
   if (T == 0) return MOTE_OK;
   const int64_t total = T * (d / 4);
   const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, 148 * 16);
-  if (pdl)
-    MOTE_CUDA_OK(launch_pdl(combine_kernel, dim3(blocks), dim3(256), 0, stream, s, y, w, perm,
-                            static_cast<const uint16_t*>(residual), T, d, k, static_cast<uint16_t*>(out_bf16),
-                            n_partials));
-  else
-    combine_kernel<<<blocks, 256, 0, stream>>>(s, y, w, perm, static_cast<const uint16_t*>(residual), T, d, k,
-                                               static_cast<uint16_t*>(out_bf16), n_partials);
+#define MOTE_COMBINE_LAUNCH(B_)                                                                                       \
+  do {                                                                                                               \
+    if (pdl)                                                                                                         \
+      MOTE_CUDA_OK(launch_pdl(combine_kernel<B_>, dim3(blocks), dim3(256), 0, stream, s, y, w, perm,                 \
+                              static_cast<const uint16_t*>(residual), T, d, k, static_cast<uint16_t*>(out_bf16),     \
+                              n_partials));                                                                          \
+    else                                                                                                             \
+      combine_kernel<B_><<<blocks, 256, 0, stream>>>(s, y, w, perm, static_cast<const uint16_t*>(residual), T, d, k, \
+                                                     static_cast<uint16_t*>(out_bf16), n_partials);                  \
+  } while (0)
+  if (n_partials <= 1) MOTE_COMBINE_LAUNCH(1);
+  else if (n_partials <= 2) MOTE_COMBINE_LAUNCH(2);
+  else if (n_partials <= 4) MOTE_COMBINE_LAUNCH(4);
+  else MOTE_COMBINE_LAUNCH(8);
+#undef MOTE_COMBINE_LAUNCH
   ++g_launch_count;
   MOTE_LAUNCH_OK();
   return MOTE_OK;

@@ -277,6 +277,16 @@ def test_short_prefill_pairs_of_gemms(mote, d, f, E, k, T, kw, bits):
     check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
 
 
+@pytest.mark.parametrize("splits,k", [(2, 1), (2, 3), (3, 2), (4, 3), (5, 1), (8, 2), (9, 3), (16, 2)])
+def test_combine_of_every_number_of_partial_sums(mote, splits, k):
+    # a shared down projection of few row tiles is cut into f / 256 parts, which the combine adds two, four or eight at a time
+    wl = synth.custom("partials", 128, 256 * splits, 4, k, 37, 8000 + 10 * splits + k)
+    master, layer_or, layer_gpu = _setup(mote, wl, TENSOR)
+    rng = np.random.default_rng(splits)
+    residual = O.f32_to_bf16_rn(rng.standard_normal((37, 128)).astype(np.float32))
+    check_forward(mote, layer_gpu, layer_or, synth.tokens(wl), residual_bits=residual)
+
+
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("path", ALL)
 def test_rtn_shared_expert_c3_decode(mote, path, bits, c3_layers):
