@@ -313,10 +313,10 @@ mote_status_t mote_stack_forward(const mote_layer_t* layers_host, int n_layers, 
  * A stage that a path folds into its neighbour reports 0: the tensor path does the combine in the
  * shared-down epilogue (stage 7); the decode path reports its prologue (Q_a(x), router, dispatch)
  * as stage 0 and its two streaming kernels, which cover the routed AND the shared expert (and, in
- * the second one, the combine), as stages 3 and 5; a short prefill (one whose shared down projection is
- * cut along K) runs the routed and the shared GEMM of a step as one launch, reported as stages 3 and 5.
- * An RTN prefill's code expansion counts into stage 6 (3 in a short prefill).  Up to 512
- * tokens Q_a(x) (stage 2) does the dispatch too.  Stages run back to back on one
+ * the second one, the combine), as stages 3 and 5; most short prefills (those whose shared down projection
+ * is cut along K) run the routed and the shared GEMM of a step as one launch, reported as stages 3 and 5.
+ * An RTN prefill's code expansion counts into the first stage that uses it (6, or 3 where the GEMMs share
+ * a launch).  Up to 512 tokens Q_a(x) (stage 2) does the dispatch too.  Stages run back to back on one
  * stream here even if mote_moe_forward overlaps some of them. */
 enum { MOTE_N_STAGES = 9 };
 mote_status_t mote_moe_forward_profile(const mote_layer_t* L, const void* x_bf16,

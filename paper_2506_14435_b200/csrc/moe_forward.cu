@@ -50,6 +50,9 @@ struct Plan {
 // the GEMM expands the codes tile by tile in shared memory (less weight traffic, more work per row tile).
 constexpr int64_t kExpandMinTokens = 768;
 constexpr int64_t kStreamAutoMaxTokens = 32;
+// Short prefills with bf16 operands for the shared expert run the routed and the shared GEMM of a step as one launch up to
+// this many multiply-adds of the shared gate projection (T * d * f): 975 tokens at 2048 x 11008.
+constexpr int64_t kPairMaxWork = 22000000000ll;
 
 static Plan make_plan(int d, int f, int E, int k, int64_t T) {
   Plan p{};
@@ -388,8 +391,9 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   // prefill with an RTN-coded shared expert and room in the workspace: expand the codes to bf16 once
   SharedMat xg = sh_gate, xu = sh_up, xd = sh_down;
   int x_bits = sh_bits;
+  const bool expands = sh_rtn && tensor && T >= kExpandMinTokens && ws_bytes >= pl.total_expanded;
   auto expand_shared = [&]() -> mote_status_t {
-    if (!(sh_rtn && tensor && T >= kExpandMinTokens && ws_bytes >= pl.total_expanded)) return MOTE_OK;
+    if (!expands) return MOTE_OK;
     char* e0 = base + pl.sh_codes_bf16;
     const size_t mat = size_t(d) * f * 2;
     ExpandArgs ea{};
@@ -401,13 +405,17 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
     x_bits = MOTE_SHARED_BF16;                     // bf16 operands; the row scales still apply
     return launch_expand_codes(ea, int64_t(d) * f, sh_bits, stream);
   };
-  // Few row tiles (the shared down projection is cut along K): neither the routed nor the shared GEMM of a step fills the
-  // SMs and both are short, so they are one launch, which also saves two.  A 64-token call of a 256 x 512 layer took
-  // 43.0 us in nine launches and takes 33.0 in seven; 1536 x 8960, 8 experts: 117 -> 107 (64 tokens), 162 -> 157 (512),
-  // 228 -> 228 (1024).  With more row tiles every GEMM fills the SMs by itself, and the shared down projection's
-  // epilogue does the combine, for which the routed one has to be complete.
+  // Few row tiles (the shared down projection is cut along K): the routed and the shared GEMM of a step both end in a
+  // partly filled round of tiles, so they are one launch, which also saves two.  Layers apart / as pairs: 256 x 512, 64
+  // tokens, 43.0 us in nine launches / 27.5 in six; 1536 x 8960, 8 experts, top-2: 116 / 99 (64 tokens), 152 / 147 (512),
+  // 200 / 194 (896), 261 / 257 (1408); 896 x 4864: 134 / 126 (1408).  A bf16 tile has three pipeline stages in a pair and
+  // four by itself, which shows once the shared GEMMs are long, hence kPairMaxWork: 2048 x 11008, 4 experts, top-1: 184 /
+  // 185 (640), 223 / 215 (896), 247 / 254 (1024), 268 / 279 (1152).  Tiles of RTN codes have three either way: 4096 x 14336,
+  // INT8, 384 tokens: 384 / 365.  With more row tiles yet, the shared down projection's epilogue does the combine, for
+  // which the routed one has to be complete.
   const int k_splits = tensor ? shared_down_k_splits(T, d, f) : 1;
-  const bool pair = tensor && k_splits > 1;
+  const bool codes = sh_rtn && !expands;
+  const bool pair = k_splits > 1 && (codes || T * int64_t(d) * f <= kPairMaxWork);
   if (pair && (st = expand_shared())) return st;
   // S4 gate/up
   TernaryGemmArgs g1{};
@@ -450,8 +458,13 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
                 : launch_shared_gateup_simt(x, sh_gate, sh_up, sh_bits, T, d, f, hs, stream);
   if (st) return st;
   stage_mark(7, stream);
-  if (pair) {
-    // the shared down projection was cut along K; its partial outputs are added by the combine
+  if (k_splits > 1) {
+    // the shared down projection is cut along K; its partial outputs are added by the combine
+    if (!pair) {
+      st = launch_shared_umma(hs, xd, SharedMat{nullptr, nullptr}, x_bits, false, T, f, d, s, tiles_shared,
+                              max_mtiles_shared, status, nullptr, stream, pdl, k_splits);
+      if (st) return st;
+    }
     stage_mark(8, stream);
     st = launch_combine(s, y, topk_w, perm, residual, T, d, k, out, stream, pdl, k_splits);
     if (st) return st;

@@ -277,6 +277,17 @@ def test_short_prefill_pairs_of_gemms(mote, d, f, E, k, T, kw, bits):
     check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
 
 
+def test_longest_short_prefill_runs_its_gemms_apart(mote):
+    # K splits of the shared down projection (two), but GEMMs too long to share a launch; a sample of the tokens
+    T = 2047
+    wl = synth.custom("apart", 384, 28672, 2, 1, T, 9100)
+    master, layer_or, layer_gpu = _setup(mote, wl, TENSOR)
+    toks = np.unique(np.concatenate([np.arange(0, T, 61), [126, 127, 128, T - 1]]))
+    check_forward(mote, layer_gpu, layer_or, synth.tokens(wl), token_subset=toks)
+    mote.mote_moe_forward(layer_gpu, bf16_tensor(synth.tokens(wl)))
+    assert mote.lib.mote_last_launch_count() == 9      # router, scan, Q_a(x), Q_a(h), four GEMMs, combine
+
+
 @pytest.mark.parametrize("splits,k", [(2, 1), (2, 3), (3, 2), (4, 3), (5, 1), (8, 2), (9, 3), (16, 2)])
 def test_combine_of_every_number_of_partial_sums(mote, splits, k):
     # a shared down projection of few row tiles is cut into f / 256 parts, which the combine adds two, four or eight at a time
