@@ -996,12 +996,26 @@ mote_status_t launch_decode_stream(const DecodeStreamArgs& p, int phase, cudaStr
     ga.hs = static_cast<uint16_t*>(p.hs); ga.tap_gate = p.tap_gate; ga.tap_up = p.tap_up;
     const int tiles = f / 8, quads = (tiles + kGuWarps - 1) / kGuWarps;
     const int max_items = tiles + std::min<int>(E, T * k) * quads;
-    // as many CTAs as are resident at once: each walks over its items, and the start of a CTA (list of experts, first
-    // loads) is paid once.  With twelve per SM in several waves: eight layers of 2048 x 11008 at 32 tokens 1326 against
-    // 1288 us, at one token 382.5 against 378; three layers at 9 tokens 353 against 330.  Up to 8 tokens with more than
-    // two items per resident CTA the waves stay: their order evens out unequal items (1536 x 8960, 8 experts, 8 tokens:
-    // 52.7 against 54.6 us).  (33 and more tokens: few CTAs fit, not measured to gain.)
-    const int per_sm = ntb == 4 ? 4 : ntb == 2 || (ntb == 1 && max_items <= 14 * sms) ? 7 : 12;
+    // As many CTAs as are resident at once, each walking over its items: the start of a CTA (list of experts, first loads)
+    // is paid once.  By registers these are, per SM, 7 / 8 / 6 (bf16, INT8, INT4) up to 8 tokens, 7 / 5 / 5 for 9 to 16 and
+    // 4 for 17 to 32.  Or waves of twelve CTAs per SM: their order evens out unequal items and a nearly empty last round.
+    // All against waves, us per layer:
+    //   17 to 32 tokens, 4: 2048 x 11008, 16 experts, 32 tokens 165 -> 161, 4 experts 95 -> 90; 1280 x 6912, 8 experts 66 -> 68.
+    //   9 to 16, where the rounds are at most two or fill the last one to 0.6 (RTN codes: or are more than four):
+    //     RTN codes, 5: INT8, 2048 x 11008, 16 / 8 / 4 experts 97 / 96 / 98 % of the time, 1536 x 8960, 8 experts 96 %; INT4 the
+    //     same within 1 %.  (7, two of them in a second round: 101 to 105 %.)  Elsewhere waves (1280 x 6912, 8 experts, 3.5 rounds:
+    //     100 to 103 %).
+    //     bf16, 7: 2048 x 5632, 4 experts 94 %, 1408 x 7040 97 %, 2048 x 11008 98 to 99 %.  Elsewhere waves (1536 x 8960, 4 experts,
+    //     2.16 rounds: 108 %; 8 and 16 experts, 3.24 and 5.4 rounds: 102 and 101 %).
+    //   up to 8, 7 for every width (INT8 8: no better than waves; INT4 6: the same within 1 %) in at most two rounds: bf16, 2048 x
+    //     11008, one token 44.1 -> 43.5; 1024 x 8192, INT8 24.1 -> 22.4; 1536 x 8960, INT4 25.8 -> 25.1; but INT8, 2048 x 11008,
+    //     16 experts 38.4 -> 39.3.  Beyond that waves (bf16, 1280 x 6912, 8 experts, 3 tokens, 2.08 rounds: 41.3, with 7: 44.4).
+    //   33 and more tokens: few CTAs fit, not measured to gain.
+    const bool rtn = p.shared_bits != 16;
+    const int resident = ntb == 4 ? 4 : ntb == 2 && rtn ? 5 : 7, round = resident * sms;
+    const bool walk = ntb == 4 || (ntb <= 2 && max_items <= 2 * round) ||
+                      (ntb == 2 && (max_items % round * 10 >= round * 6 || (rtn && max_items > 4 * round)));
+    const int per_sm = walk ? resident : 12;
     const int grid = std::min(max_items, sms * per_sm);
 #define MOTE_GU_LAUNCH(NTB_, BITS_) \
   MOTE_CUDA_OK(launch_pdl(decode_gateup_kernel<NTB_, BITS_>, dim3(grid), dim3(kGuWarps * 32), 0, stream, ga))

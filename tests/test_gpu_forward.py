@@ -227,6 +227,22 @@ def test_stream_path_17_to_32_tokens(mote, d, f, E, k, T, kw, bits):
 
 
 @pytest.mark.parametrize("bits", [16, 8, 4])
+@pytest.mark.parametrize("f,T", [
+    (512, 9),                                             # fewer gate/up items than CTAs fit
+    (8704, 12),                                           # 2176: bf16 in waves, codes in three full rounds of a walk
+    (9472, 16),                                           # 2368: waves for every width
+    (12288, 15),                                          # 3072: three rounds (bf16), more than four (codes)
+])
+def test_stream_path_9_to_16_tokens(mote, f, T, bits):
+    wl = synth.custom("grids", 64, f, 4, 2, T, 7200 + f + T, bias="zipf")
+    master, layer_or, layer_gpu = _setup(mote, wl, STREAM)
+    if bits != 16:
+        layer_or = O.quantize_shared(layer_or, bits)
+        layer_gpu = layer_gpu.quantize_shared(bits)
+    check_forward(mote, layer_gpu, layer_or, synth.tokens(wl))
+
+
+@pytest.mark.parametrize("bits", [16, 8, 4])
 @pytest.mark.parametrize("f,T", [(128, 17), (1216, 24), (4864, 32)])      # fewer steps than slices; uneven; several per slice
 def test_shared_expert_does_not_depend_on_the_routed_ones(mote, f, T, bits):
     # one expert or sixteen beside it decides how many warps a CTA of the down kernel has, not how its sums are grouped
