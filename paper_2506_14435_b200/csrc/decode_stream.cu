@@ -910,8 +910,11 @@ __device__ __forceinline__ void down_tile_done(const DecodeDownArgs& a, int tile
 // takes 106 registers, one CTA per SM, and the step is 5-10 % slower.  The 16-token 4-bit expansion
 // would spill too much under that cap.)
 // 17 to 32 tokens at 128 registers: CTAs of eight warps, two per SM, so that one streams while the other adds up, where
-// there are more than two items per SM (2048 x 11008, 16 experts, 32 tokens: kernel 86 -> 74 us; four warps: the same);
-// CTAs of sixteen below that (896 x 4864, 4 experts, 17 tokens: layer 35.0 against 36.1 us).  Up to 16 tokens eight warps
+// there are more than two items per SM (2048 x 11008, 16 experts, 32 tokens: kernel 86 -> 74 us; four warps: the same).  From
+// one to two items per SM the longest tile decides: CTAs of eight warps up to 40 000 bits per shared row (layers of 32 tokens
+// with sixteen / eight warps: 896 x 4864, 4 experts, INT8 48.1 / 45.9 us, INT4 48.7 / 45.8; 512 x 2048, bf16 33.1 / 31.7; 256 x
+// 512, 16 experts 30.4 / 27.6), of sixteen above (896 x 4864, bf16, 17 tokens 38.8 / 40.2; 1024 x 8192, 2 experts, INT8 37.4 / 41.4;
+// 2048 x 11008, 1 expert, INT4, 32 tokens 88.6 / 91.3).  Up to 16 tokens eight warps
 // are slower (382 -> 460 us per eight layers of one token: a shared tile's 352 KB come in too slowly).
 template <int NTB, int kShBits, int kDownWarps>
 __global__ void __launch_bounds__(kDownWarps * 32,
@@ -1044,7 +1047,8 @@ mote_status_t launch_decode_stream(const DecodeStreamArgs& p, int phase, cudaStr
   da.hs = static_cast<const uint16_t*>(p.hs); da.y = p.y; da.s = p.s; da.tap_down = p.tap_down;
   const int tiles = d / 16;
   const int max_items = tiles + std::min<int>(E, T * k) * tiles;
-  const int warps = ntb == 4 && max_items > 2 * sms ? 8 : 16;
+  // see decode_down_kernel; f * bits: bits of a shared row
+  const int warps = ntb == 4 && (max_items > 2 * sms || (max_items > sms && f * p.shared_bits <= 40000)) ? 8 : 16;
   const int grid = std::min(max_items, sms * (48 / warps));
   const size_t smem = size_t(kDownSlices) * ntb * 4 * 32 * sizeof(float);
   static PerDeviceOnce down_attr16, down_attr8, down_attr4;

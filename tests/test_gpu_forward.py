@@ -214,6 +214,7 @@ def test_rtn_shared_expert(mote, d, f, E, k, T, kw, path, bits):
 @pytest.mark.parametrize("bits", [16, 8, 4])
 @pytest.mark.parametrize("d,f,E,k,T,kw", [
     (256, 512, 4, 1, 20, {}),                             # few down items: sixteen warps each
+    (512, 2560, 4, 2, 21, {}),                            # 160 down items: sixteen warps where the rows are bf16, eight for codes
     (1024, 256, 8, 2, 17, {}),                            # many: eight warps, one reduction step among them
     (1088, 4864, 8, 2, 32, dict(bias="zipf")),            # ... and 19 uneven steps, experts of one to four token tiles
 ])
