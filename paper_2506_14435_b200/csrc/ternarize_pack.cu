@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(256) pack_codes_kernel(const void* __restrict_
       for (int j = 0; j < kPer; ++j) {
         const float x = __uint_as_float(bits[r * kPer + j]);
         if (x > half) out += 1u << (2 * j);
-        if (x < -half) out -= 1u << (2 * j);
+        if (!(x >= -half)) out -= 1u << (2 * j);           // a NaN too, as the clamp of the quotient from below would give
       }
       if ((r * 32 + lane) * kPer < left) {
         if (kBf16) reinterpret_cast<uint16_t*>(packed)[v * 64 + r * 32 + lane] = (uint16_t)out;

@@ -72,6 +72,22 @@ def test_ternarize_pack_exact_sum_paths_and_thresholds(mote, shape, zeros, sprea
     assert np.array_equal(packed.cpu().numpy(), O.pack_codes(codes))
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_ternarize_pack_non_finite_weights_stay_where_they_are(mote, dtype):
+    # left out of alpha; infinities saturate, a NaN takes the code that max(NaN, -1) gives
+    W = torch.from_numpy(_randn((40, 528), 23, 0.02).astype(np.float32)).to(dtype)
+    finite = W.clone()
+    at = [(0, 0), (0, 7), (11, 300), (39, 527)]
+    for (i, j), v in zip(at, (float("nan"), float("inf"), -float("inf"), float("nan"))):
+        W[i, j], finite[i, j] = v, 0.0
+    codes, alpha = O.ternarize(finite.float().numpy())
+    for (i, j), c in zip(at, (-1, 1, -1, -1)):
+        codes[i, j] = c
+    packed, a = mote.mote_ternarize_pack(W.cuda())
+    assert a.item() == alpha
+    assert np.array_equal(packed.cpu().numpy(), O.pack_codes(codes))
+
+
 def test_ternarize_pack_bf16_input(mote):
     Wb = O.f32_to_bf16_rn(_randn((96, 320), 5, 0.02).astype(np.float32))
     codes, alpha = O.ternarize(O.bf16_to_f32(Wb))
