@@ -136,12 +136,35 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(sm)}
 
 
+def gemms_in_pairs(launches: int, T: int, shared_bits: int) -> bool:
+    """Whether a tensor-path layer call of so many launches ran the routed and the shared GEMM of a step as one (most short
+    prefills do): router, Q_a(x), gate/up, Q_a(h), down and combine, beside the dispatch scan of more than 512 tokens and
+    the code expansion of an RTN-coded shared expert from 768 tokens on.  Apart they are at least one launch more."""
+    return launches - (T > 512) - (shared_bits != 16 and T >= 768) == 6
+
+
+def gemm_ops(wl: synth.Workload, stage: str) -> float:
+    """Multiply and add counted as two; int8 in the routed stages, bf16 in the shared ones."""
+    rows = wl.T if stage.startswith("shared") else wl.T * wl.k
+    return (4.0 if "gateup" in stage else 2.0) * rows * wl.d * wl.f
+
+
+SHARED_STAGE = {"gateup_ternary": "shared_gateup", "down_ternary": "shared_down"}
+
+
+def mixed_peak(wl: synth.Workload, stage: str, int8_tops: float, bf16_tflops: float) -> float:
+    """The rate of a pair of GEMMs whose routed part runs at the int8 peak and whose shared part at the bf16 one."""
+    r, sh = gemm_ops(wl, stage), gemm_ops(wl, SHARED_STAGE[stage])
+    return (r + sh) / (r / int8_tops + sh / bf16_tflops)
+
+
 def stage_work(wl: synth.Workload, stage: str, stream_path: bool, experts_touched: float, shared_bits: int = 16,
-               peaks: dict | None = None):
-    """Algorithmic work of one launch of a stage: (amount, kind), kind 'int8' | 'bf16' | 'bytes'.
-    On the decode path (and in a short prefill, whose GEMMs run in pairs) the gate/up and down stages each
-    cover the routed AND the shared expert and are bound by the weight bytes they stream: 2-bit codes of the experts that received tokens plus
-    the shared matrices (bf16, or RTN codes of shared_bits bits)."""
+               peaks: dict | None = None, paired: bool = False):
+    """Algorithmic work of one launch of a stage: (amount, kind), kind 'int8' | 'bf16' | 'mixed' | 'bytes'.
+    On the decode path the gate/up and down stages each cover the routed AND the shared expert and
+    are bound by the weight bytes they stream: 2-bit codes of the experts that received tokens plus
+    the shared matrices (bf16, or RTN codes of shared_bits bits).  In a short prefill whose GEMMs run in pairs they
+    cover both too, and are bound by those bytes or by the tensor work of both ('mixed')."""
     P, T, d, f = wl.T * wl.k, wl.T, wl.d, wl.f
     sh_bytes = shared_bits / 8.0
     if stream_path:
@@ -151,14 +174,20 @@ def stage_work(wl: synth.Workload, stage: str, stream_path: bool, experts_touche
             return experts_touched * f * d / 4 + f * d * sh_bytes, "bytes"
     # the four GEMMs: tensor work, or -- with few tokens -- the bytes they must move, whichever takes
     # longer at the peaks (a short prefill streams the weights once and is bound by that)
-    gemm = {"gateup_ternary": (2.0 * P * d * 2 * f, "int8", experts_touched * 2 * f * d / 4 + P * d + P * f * 2.0),
-            "down_ternary": (2.0 * P * f * d, "int8", experts_touched * f * d / 4 + P * f + P * d * 4.0),
-            "shared_gateup": (2.0 * T * d * 2 * f, "bf16", 2.0 * f * d * sh_bytes + T * d * 2.0 + T * f * 2.0),
-            "shared_down": (2.0 * T * f * d, "bf16", f * d * sh_bytes + T * f * 2.0 + T * d * 2.0)}
-    if stage in gemm:
-        ops, kind, nbytes = gemm[stage]
+    gemm_bytes = {"gateup_ternary": experts_touched * 2 * f * d / 4 + P * d + P * f * 2.0,
+                  "down_ternary": experts_touched * f * d / 4 + P * f + P * d * 4.0,
+                  "shared_gateup": 2.0 * f * d * sh_bytes + T * d * 2.0 + T * f * 2.0,
+                  "shared_down": f * d * sh_bytes + T * f * 2.0 + T * d * 2.0}
+    if stage in gemm_bytes:
+        ops, nbytes = gemm_ops(wl, stage), gemm_bytes[stage]
+        kind = "bf16" if stage.startswith("shared") else "int8"
+        if paired and stage in SHARED_STAGE:
+            ops += gemm_ops(wl, SHARED_STAGE[stage])
+            nbytes += gemm_bytes[SHARED_STAGE[stage]]
+            kind = "mixed"
         if peaks is not None:
-            t_ops = ops / ((peaks["int8_tops"] if kind == "int8" else peaks["bf16_tflops"]) * 1e12)
+            rate = {"int8": peaks["int8_tops"], "bf16": peaks["bf16_tflops"]}
+            t_ops = ops / ((mixed_peak(wl, stage, *rate.values()) if kind == "mixed" else rate[kind]) * 1e12)
             if nbytes / (peaks["hbm_gbs"] * 1e9) > t_ops:
                 return nbytes, "bytes"
         return ops, kind
@@ -303,6 +332,7 @@ def measure(ls: LayerSet, wl: synth.Workload, args, steps: int | None, rank: int
         taps = layer.alloc_taps(wl.T, names=["offsets"])
         nxt = mote.mote_moe_forward(layer, mote.mote_rms_norm(cur) if is_stack else cur,
                                     residual=cur if is_stack else None, taps=taps)
+        layer_launches = mote.lib.mote_last_launch_count()
         touched.append(int((taps["offsets"][1:] - taps["offsets"][:-1] > 0).sum().item()))
         cur = nxt
     experts_touched = sum(touched) / len(touched)
@@ -365,8 +395,7 @@ def measure(ls: LayerSet, wl: synth.Workload, args, steps: int | None, rank: int
     # chain of programmatic dependent launches): the stages this path folds into a neighbour launch
     # nothing, so what they show is that cost alone.  It is taken off the stages that do launch.
     n_l0 = len(layers)
-    # a short prefill runs the routed and the shared GEMM of a step as one launch: the shared stages launch nothing
-    paired = not stream_path and max(stage_raw["shared_gateup"], stage_raw["shared_down"]) / n_l0 < 4e-3
+    paired = not stream_path and gemms_in_pairs(layer_launches, wl.T, args.shared_bits)    # the shared stages launch nothing
     folded = (("dispatch", "quant_x", "shared_gateup", "shared_down", "combine") if stream_path
               else ("shared_gateup", "shared_down") if paired else ("combine",))
     event_ms = min(stage_raw[k_] for k_ in folded) / n_l0
@@ -396,7 +425,7 @@ def measure(ls: LayerSet, wl: synth.Workload, args, steps: int | None, rank: int
     sustained = total_ms >= SUSTAINED_MIN_MS
     n_l = len(layers)
     dom = max(stage_ms, key=stage_ms.get)
-    work, kind = stage_work(wl, dom, stream_path or paired, experts_touched, args.shared_bits, peaks)
+    work, kind = stage_work(wl, dom, stream_path, experts_touched, args.shared_bits, peaks, paired)
     dur_s = stage_ms[dom] * 1e-3 / n_l                  # average duration of one launch of that kernel
     from paper_2506_14435_b200 import traffic
     label = workload_label(wl)
@@ -410,6 +439,12 @@ def measure(ls: LayerSet, wl: synth.Workload, args, steps: int | None, rank: int
                                  ("sustained figure (timed region of %.0f ms)" % total_ms if sustained else "burst figure")),
                     peak_burst=peaks["int8_tops"], peak_sustained=peaks["int8_tops_sustained"],
                     peak_2x_bf16_burst=2.0 * peaks["bf16_tflops"], frac_of_nominal=work / dur_s / 1e12 / NOMINAL["int8_tops"])
+    elif kind == "mixed":
+        mix = [peaks["int8_tops_sustained"], peaks["bf16_tflops_sustained"]] if sustained else [peaks["int8_tops"], peaks["bf16_tflops"]]
+        roof = dict(bound="tensor", achieved=work / dur_s / 1e12, peak=mixed_peak(wl, dom, *mix), unit="TOP/s",
+                    peak_source=f"of measured, routed work at the int8 MMA-only loop's rate and shared work at cuBLAS bf16's "
+                                f"({peaks['source']}), " + ("sustained" if sustained else "burst"),
+                    frac_of_nominal=work / dur_s / 1e12 / mixed_peak(wl, dom, NOMINAL["int8_tops"], NOMINAL["bf16_tflops"]))
     else:
         peak = peaks["bf16_tflops_sustained"] if sustained else peaks["bf16_tflops"]
         roof = dict(bound="tensor", achieved=work / dur_s / 1e12, peak=peak, unit="TFLOP/s",

@@ -72,3 +72,31 @@ def test_replica_command_is_one_rank_per_gpu_on_the_loopback_address():
     assert "--nproc-per-node=4" in cmd and "--nnodes=1" in cmd
     assert cmd[cmd.index("--master-addr") + 1] == "127.0.0.1" and cmd[cmd.index("--master-port") + 1] == "29555"
     assert cmd[-4:] == ["--gpus", "4", "--steps", "7"]
+
+
+def test_paired_gemms_are_bound_by_bytes_or_by_the_tensor_work_of_both():
+    import bench
+    from workloads import synth
+    peaks = dict(hbm_gbs=6500.0, int8_tops=4500.0, bf16_tflops=1700.0)
+    wl = synth.custom("pair", 896, 4864, 4, 2, 64, 1)
+    amount, kind = bench.stage_work(wl, "gateup_ternary", False, 4.0, 16, peaks, paired=True)
+    weights = 896 * 4864 * 2 * (4 / 4 + 2)                      # four experts at two bits and the shared one at sixteen
+    assert kind == "bytes" and weights < amount < 1.1 * weights
+    wl = wl.with_T(1500)                                        # 13 us of int8 and 15 us of bf16 work; 6 us of bytes
+    for stage, n_mat in (("gateup_ternary", 2), ("down_ternary", 1)):
+        amount, kind = bench.stage_work(wl, stage, False, 4.0, 16, peaks, paired=True)
+        one = 2.0 * 1500 * 896 * 4864 * n_mat
+        assert kind == "mixed" and amount == one * (2 + 1)
+        seconds = amount / (bench.mixed_peak(wl, stage, 4500.0, 1700.0) * 1e12)
+        assert abs(seconds - (2 * one / 4500e12 + one / 1700e12)) < 1e-9 * seconds
+    # by themselves, and on the decode path, the stages are what they were
+    assert bench.stage_work(wl, "gateup_ternary", False, 4.0, 16, peaks) == (4.0 * 3000 * 896 * 4864, "int8")
+    assert bench.stage_work(wl, "shared_down", False, 4.0, 16, peaks) == (2.0 * 1500 * 896 * 4864, "bf16")
+    assert bench.stage_work(wl, "down_ternary", True, 4.0, 8, peaks) == (896 * 4864 * 2.0, "bytes")
+
+
+def test_pairs_are_told_by_the_number_of_launches():
+    import bench
+    for T, bits, apart in ((64, 16, 8), (512, 8, 8), (513, 16, 9), (767, 4, 9), (768, 4, 10), (1152, 16, 9), (1152, 8, 10)):
+        assert bench.gemms_in_pairs(apart - 2, T, bits) and not bench.gemms_in_pairs(apart, T, bits)
+        assert not bench.gemms_in_pairs(apart - 1, T, bits)     # no K splits: the combine is folded into the shared down GEMM
