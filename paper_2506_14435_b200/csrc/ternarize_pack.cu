@@ -20,9 +20,8 @@ namespace mote {
 constexpr int kBins = 256;
 
 // Exact sum of |w|: every thread keeps ONE 64-bit fixed-point accumulator in units of 2^(base - 150).
-// An element with exponent e in [base, base + 31] adds significand << (e - base), below 2^55, so some
-// five hundred elements fit before a flush is needed;
-// the grid gives a thread far fewer, and the flush is made anyway every 256 additions (and when a larger element moves the window up).  A flush adds
+// An element with exponent e in [base, base + 31] adds significand << (e - base), below 2^55, so 511 elements
+// fit; the accumulator is flushed after 256 to 271 of them (and when a larger element moves the window up).  A flush adds
 // the low 32 bits to bin `base` and the high 32 bits to bin `base + 32` (whose unit is 2^32 times
 // larger): exact, and every bin stays far below 2^64.  The rare element outside the window goes
 // straight to the bin of its own exponent.  All of it is integer addition, so neither the choice of

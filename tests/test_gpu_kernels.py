@@ -67,6 +67,7 @@ def test_ternarize_pack_exact_sum_paths_and_thresholds(mote, shape, zeros, sprea
         if O.ternarize(W)[1] == alpha:
             break
     codes, alpha = O.ternarize(W)
+    assert np.float32(alpha) / np.float32(2) in W, "no weight on alpha/2"
     packed, a = mote.mote_ternarize_pack(torch.from_numpy(W).cuda())
     assert a.item() == alpha
     assert np.array_equal(packed.cpu().numpy(), O.pack_codes(codes))

@@ -29,6 +29,17 @@ def test_ternarize_pack_larger_than_l2(mote):
     assert np.array_equal(packed.cpu().numpy(), O.pack_codes(codes))
 
 
+# A warp takes items of 512 weights.  148 x 32 warps: more than sixteen items each (an accumulator is put away every
+# sixteen), and one or two each with a ragged last one.
+@pytest.mark.parametrize("m,n", [(4800, 8192), (1201, 2064)])
+def test_ternarize_pack_bf16_many_items_per_warp(mote, m, n):
+    Wb = O.f32_to_bf16_rn(_gauss((m, n), 17, 0.02).astype(np.float32))
+    codes, alpha = O.ternarize(O.bf16_to_f32(Wb))
+    packed, a = mote.mote_ternarize_pack(bf16_tensor(Wb))
+    assert a.item() == alpha
+    assert np.array_equal(packed.cpu().numpy(), O.pack_codes(codes))
+
+
 @pytest.mark.parametrize("bits", [8, 4])
 def test_rtn_quant_larger_than_l2(mote, bits):
     Wb = O.f32_to_bf16_rn(_gauss((8192, 10240), 12 + bits, 0.02).astype(np.float32))     # 168 MB of bf16
