@@ -341,8 +341,13 @@ __device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_
   item_k_range<TR::kGateUp>(a, item, kb, ke);
   for (int ks = kb; ks < ke; ++ks, ++step) {
     if ((step & 1u) == (uint32_t)group) {
-      const bool ok = mbar_wait(smem_u32(&bars->full_p[q.stage]), q.phase, abort_flag) &&
-                      mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, abort_flag);
+      // In this order: once the MMA has left the operand stage, the step kStages back is done, so the code stage's last
+      // use (kStagesP >= kStages steps back) has completed its phase.  Asked for first, full_p could still be in the phase
+      // before that one, which its parity does not tell from the one wanted: with three code stages (INT8) a stage's
+      // steps fall to the two groups in turn, and this group has not waited for the other's.
+      static_assert(kStagesP >= S, "a code stage must not come round before its operand stage");
+      const bool ok = mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, abort_flag) &&
+                      mbar_wait(smem_u32(&bars->full_p[q.stage]), q.phase, abort_flag);
       if (!__all_sync(0xffffffffu, ok)) return false;
       const uint8_t* src = genP + q.stage * kStageP;
       uint8_t* dst = genB + p.stage * kStageB;
