@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kDispatchThreads) dispatch_kernel(const int32_
 // ------------------------------------------------------------------------------------------------
 // Block-wise dispatch for long prefills.  The router leaves, for every block of kRouteBlockTokens
 // tokens, the number of its pairs per expert (blk_hist[E][blk_stride(n_blk)]).  This kernel turns
-// them into
+// them into (tr, ts: rows per tile of the two tables)
 //   offsets[E+1]                      first sorted row of every expert
 //   blk_base[E][blk_stride(n_blk)]    first sorted row of the block's pairs of that expert
 // (experts outermost, blocks in order: the same stable order as above) and writes the tile tables.
@@ -145,8 +145,8 @@ __device__ __forceinline__ void load_counts(const int32_t* __restrict__ row, int
 __global__ void __launch_bounds__(kDispatchThreads) dispatch_scan_kernel(const int32_t* __restrict__ blk_hist, int n_blk,
                                                                          int E, int32_t* __restrict__ offsets,
                                                                          int32_t* __restrict__ blk_base,
-                                                                         int4* __restrict__ tiles_routed,
-                                                                         int4* __restrict__ tiles_shared, int T) {
+                                                                         int4* __restrict__ tiles_routed, int tr,
+                                                                         int4* __restrict__ tiles_shared, int ts, int T) {
   __shared__ int s_count[MOTE_MAX_EXPERTS];
   __shared__ int s_first[MOTE_MAX_EXPERTS];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -182,14 +182,14 @@ __global__ void __launch_bounds__(kDispatchThreads) dispatch_scan_kernel(const i
     int n = 0, run = 0;
     for (int e = 0; e < E; ++e) {
       const int cnt = s_count[e];
-      for (int r = 0; r < cnt; r += 128) tiles_routed[1 + n++] = make_int4(e, run + r, min(128, cnt - r), 0);
+      for (int r = 0; r < cnt; r += tr) tiles_routed[1 + n++] = make_int4(e, run + r, min(tr, cnt - r), 0);
       run += cnt;
     }
     tiles_routed[0] = make_int4(n, 0, 0, 0);
   }
   if (tiles_shared) {
-    const int n = (T + 127) / 128;
-    for (int i = tid; i < n; i += kDispatchThreads) tiles_shared[1 + i] = make_int4(0, i * 128, min(128, T - i * 128), 0);
+    const int n = (T + ts - 1) / ts;
+    for (int i = tid; i < n; i += kDispatchThreads) tiles_shared[1 + i] = make_int4(0, i * ts, min(ts, T - i * ts), 0);
     if (tid == 0) tiles_shared[0] = make_int4(n, 0, 0, 0);
   }
   __syncthreads();
@@ -230,9 +230,10 @@ __global__ void __launch_bounds__(kDispatchThreads) dispatch_scan_kernel(const i
 }
 
 mote_status_t launch_dispatch_scan(const int32_t* blk_hist, int n_blk, int E, int32_t* offsets, int32_t* blk_base,
-                                   int4* tiles_routed, int4* tiles_shared, int64_t T, cudaStream_t stream) {
+                                   int4* tiles_routed, int cg_routed, int4* tiles_shared, int cg_shared, int64_t T,
+                                   cudaStream_t stream) {
   MOTE_CUDA_OK(launch_pdl(dispatch_scan_kernel, dim3(1), dim3(kDispatchThreads), 0, stream, blk_hist, n_blk, E, offsets,
-                          blk_base, tiles_routed, tiles_shared, (int)T));
+                          blk_base, tiles_routed, 128 * cg_routed, tiles_shared, 128 * cg_shared, (int)T));
   ++g_launch_count;
   MOTE_LAUNCH_OK();
   return MOTE_OK;

@@ -276,9 +276,6 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   auto* status = reinterpret_cast<uint32_t*>(base + pl.status);
   auto* tiles_routed = reinterpret_cast<int4*>(base + pl.tiles_routed);
   auto* tiles_shared = reinterpret_cast<int4*>(base + pl.tiles_shared);
-  const int max_mtiles_routed = (int)(P / 128 + E);
-  const int max_mtiles_shared = (int)((T + 127) / 128);
-
   const bool tensor_ok = (d % 128 == 0) && (f % 128 == 0);
   const bool stream_ok = decode_stream_supported(d, f, E, k, T);
   int path = L->path;
@@ -347,6 +344,24 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
     return MOTE_OK;
   }
 
+  const bool expands = sh_rtn && tensor && T >= kExpandMinTokens && ws_bytes >= pl.total_expanded;   // see expand_shared
+  // Few row tiles (the shared down projection is cut along K): the routed and the shared GEMM of a step both end in a
+  // partly filled round of tiles, so they are one launch, which also saves two.  Layers apart / as pairs: 256 x 512, 64
+  // tokens, 43.0 us in nine launches / 27.5 in six; 1536 x 8960, 8 experts, top-2: 116 / 99 (64 tokens), 152 / 147 (512),
+  // 200 / 194 (896), 261 / 257 (1408); 896 x 4864: 134 / 126 (1408).  A bf16 tile has three pipeline stages in a pair and
+  // four by itself, which shows once the shared GEMMs are long, hence kPairMaxWork: 2048 x 11008, 4 experts, top-1: 184 /
+  // 185 (640), 223 / 215 (896), 247 / 254 (1024), 268 / 279 (1152).  Tiles of RTN codes have three either way: 4096 x 14336,
+  // INT8, 384 tokens: 384 / 365.  With more row tiles yet, the shared down projection's epilogue does the combine, for
+  // which the routed one has to be complete.
+  const int k_splits = tensor ? shared_down_k_splits(T, d, f) : 1;
+  const bool codes = sh_rtn && !expands;
+  const bool pair = k_splits > 1 && (codes || T * int64_t(d) * f <= kPairMaxWork);
+  // CTAs per tile of the GEMMs that run apart (codes that the GEMM expands to bf16 have no kernel for pairs of CTAs)
+  const int cg_routed = tensor && !pair ? routed_ctas_per_tile(P, E, d, f) : 1;
+  const int cg_shared = tensor && !pair && !codes ? shared_ctas_per_tile(T, d, f, k_splits) : 1;
+  const int max_mtiles_routed = (int)(P / (128 * cg_routed) + E);
+  const int max_mtiles_shared = (int)((T + 128 * cg_shared - 1) / (128 * cg_shared));
+
   mote_status_t st;
   // device status word: cleared by the router kernel where the tensor-core router runs (one
   // operation less on the stream), else by a memset
@@ -366,7 +381,8 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   stage_mark(1, stream);
   const bool inline_scan = blockwise && n_blk <= kInlineScanBlocks;   // few blocks: done by the CTAs of Q_a(x)
   st = inline_scan ? MOTE_OK
-       : blockwise ? launch_dispatch_scan(blk_hist, n_blk, E, offsets, blk_base, tiles_routed, tiles_shared, T, stream)
+       : blockwise ? launch_dispatch_scan(blk_hist, n_blk, E, offsets, blk_base, tiles_routed, cg_routed, tiles_shared, cg_shared, T,
+                                          stream)
                    : launch_dispatch(topk_idx, P, E, offsets, perm, inv, tensor ? tiles_routed : nullptr,
                                    tensor ? tiles_shared : nullptr, T, stream);
   if (st) return st;
@@ -378,6 +394,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   if (blockwise) {
     if (inline_scan) {
       qa.blk_hist = blk_hist; qa.offsets_out = offsets; qa.tiles_routed = tiles_routed; qa.tiles_shared = tiles_shared;
+      qa.cg_routed = cg_routed; qa.cg_shared = cg_shared;
     } else {
       qa.blk_base = blk_base;
     }
@@ -391,7 +408,6 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   // prefill with an RTN-coded shared expert and room in the workspace: expand the codes to bf16 once
   SharedMat xg = sh_gate, xu = sh_up, xd = sh_down;
   int x_bits = sh_bits;
-  const bool expands = sh_rtn && tensor && T >= kExpandMinTokens && ws_bytes >= pl.total_expanded;
   auto expand_shared = [&]() -> mote_status_t {
     if (!expands) return MOTE_OK;
     char* e0 = base + pl.sh_codes_bf16;
@@ -405,17 +421,6 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
     x_bits = MOTE_SHARED_BF16;                     // bf16 operands; the row scales still apply
     return launch_expand_codes(ea, int64_t(d) * f, sh_bits, stream);
   };
-  // Few row tiles (the shared down projection is cut along K): the routed and the shared GEMM of a step both end in a
-  // partly filled round of tiles, so they are one launch, which also saves two.  Layers apart / as pairs: 256 x 512, 64
-  // tokens, 43.0 us in nine launches / 27.5 in six; 1536 x 8960, 8 experts, top-2: 116 / 99 (64 tokens), 152 / 147 (512),
-  // 200 / 194 (896), 261 / 257 (1408); 896 x 4864: 134 / 126 (1408).  A bf16 tile has three pipeline stages in a pair and
-  // four by itself, which shows once the shared GEMMs are long, hence kPairMaxWork: 2048 x 11008, 4 experts, top-1: 184 /
-  // 185 (640), 223 / 215 (896), 247 / 254 (1024), 268 / 279 (1152).  Tiles of RTN codes have three either way: 4096 x 14336,
-  // INT8, 384 tokens: 384 / 365.  With more row tiles yet, the shared down projection's epilogue does the combine, for
-  // which the routed one has to be complete.
-  const int k_splits = tensor ? shared_down_k_splits(T, d, f) : 1;
-  const bool codes = sh_rtn && !expands;
-  const bool pair = k_splits > 1 && (codes || T * int64_t(d) * f <= kPairMaxWork);
   if (pair && (st = expand_shared())) return st;
   // S4 gate/up
   TernaryGemmArgs g1{};
@@ -427,7 +432,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   st = pair     ? launch_umma_pair(g1, true, tiles_routed, max_mtiles_routed, rowsum_x, reinterpret_cast<uint32_t*>(beta_h), x,
                                    xg, xu, x_bits, T, hs, tiles_shared, max_mtiles_shared, status, stream, pdl, 1)
        : tensor ? launch_ternary_umma(g1, true, tiles_routed, max_mtiles_routed, rowsum_x,
-                                      reinterpret_cast<uint32_t*>(beta_h), status, stream, pdl)
+                                      reinterpret_cast<uint32_t*>(beta_h), status, stream, pdl, cg_routed)
                 : launch_ternary_gateup_simt(g1, stream);
   if (st) return st;
   stage_mark(4, stream);
@@ -446,7 +451,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   st = pair     ? launch_umma_pair(g2, false, tiles_routed, max_mtiles_routed, rowsum_h, nullptr, hs, xd,
                                    SharedMat{nullptr, nullptr}, x_bits, T, s, tiles_shared, max_mtiles_shared, status, stream,
                                    pdl, k_splits)
-       : tensor ? launch_ternary_umma(g2, false, tiles_routed, max_mtiles_routed, rowsum_h, nullptr, status, stream, pdl)
+       : tensor ? launch_ternary_umma(g2, false, tiles_routed, max_mtiles_routed, rowsum_h, nullptr, status, stream, pdl, cg_routed)
                 : launch_ternary_down_simt(g2, stream);
   if (st) return st;
   stage_mark(6, stream);
@@ -454,7 +459,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   if (!pair && (st = expand_shared())) return st;
   st = pair     ? MOTE_OK
        : tensor ? launch_shared_umma(x, xg, xu, x_bits, true, T, d, f, hs, tiles_shared, max_mtiles_shared,
-                                     status, nullptr, stream, pdl)
+                                     status, nullptr, stream, pdl, 1, cg_shared)
                 : launch_shared_gateup_simt(x, sh_gate, sh_up, sh_bits, T, d, f, hs, stream);
   if (st) return st;
   stage_mark(7, stream);
@@ -462,7 +467,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
     // the shared down projection is cut along K; its partial outputs are added by the combine
     if (!pair) {
       st = launch_shared_umma(hs, xd, SharedMat{nullptr, nullptr}, x_bits, false, T, f, d, s, tiles_shared,
-                              max_mtiles_shared, status, nullptr, stream, pdl, k_splits);
+                              max_mtiles_shared, status, nullptr, stream, pdl, k_splits, cg_shared);
       if (st) return st;
     }
     stage_mark(8, stream);
@@ -474,7 +479,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
     CombineArgs cb{y, topk_w, perm, residual, out, k};
     st = launch_shared_umma(hs, xd, SharedMat{nullptr, nullptr}, x_bits, false, T, f, d,
                             (taps && taps->shared_out) ? s : nullptr, tiles_shared, max_mtiles_shared, status, &cb,
-                            stream, pdl);
+                            stream, pdl, 1, cg_shared);
     if (st) return st;
     stage_mark(8, stream);
   } else {

@@ -56,20 +56,35 @@ __device__ __forceinline__ void u4x8_to_bf16x2(uint32_t w, uint32_t (&e)[4]) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// pdl: as a programmatic dependent; cluster: CTAs per thread-block cluster (1: none)
 template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                     Args... args) {
+static inline cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                    bool pdl, int cluster, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  unsigned n = 0;
+  if (pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                     Args... args) {
+  return launch_ex(kernel, grid, block, smem, stream, true, 1, args...);
 }
 
 constexpr float kEpsScale = 1e-5f;  // lower clamp of alpha (Eq. 9) and beta (Eq. 8)
@@ -231,28 +246,58 @@ __device__ __forceinline__ float glu_h(int acc_g, int acc_u, float c_g, float c_
 //   s'  = fl(g * rcp.approx(den'))  (rcp: <= 2^-23, product 2^-24) vs s = fl(g / den) -> <= 1.0e-6
 //   h'  = fl(u * s')                                             vs h  -> <= 1.12e-6 < 19 ulp
 // bf16_rn(h') == bf16_rn(h) unless h' lies within 19 fp32 ulps of the midpoint between two bf16
-// values; the flag is raised within 32 ulps of a midpoint (low 16 bits in [0x7FE0, 0x8020]), and
-// for |t| > 64 where the clamp, overflow or gradual underflow could make the two differ more.
-// Flagged elements (about 0.1 %) are recomputed with glu_h.  The caller must also send rows with
-// c_g * c_u <= 1e-12 to glu_h (h' could be subnormal there).
+// values; such elements (low 16 bits in [0x7FE8, 0x8018]: within 24 ulps) and those with |t| > 64, where the clamp,
+// overflow or gradual underflow could make the two differ more, are to be recomputed with glu_h (0.07 %).  The caller must also
+// send rows with c_g * c_u <= 1e-12 to glu_h (h' could be subnormal there).
+__device__ __forceinline__ uint32_t glu_midpoint_key(float h) { return (__float_as_uint(h) << 16) + 0x80180000u; }
+constexpr uint32_t kGluMidpointKeys = 0x00300000u;      // keys up to here: near a midpoint (one shift-and-add to test)
+constexpr float kGluMaxT = 64.0f;
+
+// Two floats at a time (each lane of the pair rounds as the scalar instruction does; half the issue slots).
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ uint64_t f32x2_bits(uint32_t lo, uint32_t hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// h' of two neighbouring elements, and the larger |t| of the two.
 // It works on raw accumulators that still carry the token's row sum (code + 1 storage): `bias` is
 // 0x4B400000 - rowsum, so that fl32(acc - rowsum) costs one integer add and one subtract per value
-// ((acc - rowsum) + 0x4B400000 == acc + bias in 32-bit arithmetic; see i2f_small).
-__device__ __forceinline__ float glu_h_fast_biased(uint32_t raw_g, uint32_t raw_u, uint32_t bias, float c_g, float c_u,
-                                                   bool& redo) {
-  const float g = __fmul_rn(__fsub_rn(__uint_as_float(raw_g + bias), kMagic), c_g);
-  const float u = __fmul_rn(__fsub_rn(__uint_as_float(raw_u + bias), kMagic), c_u);
-  const float t = __fmul_rn(-g, 1.4426950408889634f);
-  float e, rc;
+// ((acc - rowsum) + 0x4B400000 == acc + bias in 32-bit arithmetic; see i2f_small).  c_g, c_u: the scale, in both halves.
+__device__ __forceinline__ void glu_h2_fast_biased(uint32_t raw_g0, uint32_t raw_g1, uint32_t raw_u0, uint32_t raw_u1,
+                                                   uint32_t bias, uint64_t c_g, uint64_t c_u, float& h0, float& h1, float& t_abs) {
+  const uint64_t minus_magic = f32x2(-kMagic, -kMagic), one = f32x2(1.0f, 1.0f);
+  const uint64_t minus_log2e = f32x2(-1.4426950408889634f, -1.4426950408889634f);
+  const uint64_t g = mul_f32x2(add_f32x2(f32x2_bits(raw_g0 + bias, raw_g1 + bias), minus_magic), c_g);
+  const uint64_t u = mul_f32x2(add_f32x2(f32x2_bits(raw_u0 + bias, raw_u1 + bias), minus_magic), c_u);
+  float t0, t1, e0, e1, d0, d1, r0, r1;
+  unpack_f32x2(mul_f32x2(g, minus_log2e), t0, t1);
   // .ftz: single instructions; with |t| <= 64 neither the operands nor the results are subnormal
   // (a subnormal t is flushed to 0, where 2^t = 1 to well within the error budget)
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t));
-  const float den = __fadd_rn(1.0f, e);
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(den));
-  const float h = __fmul_rn(u, __fmul_rn(g, rc));
-  // low 16 bits in [0x7FE0, 0x8020], tested in the upper half of a word: one shift-and-add, one compare
-  redo = ((__float_as_uint(h) << 16) + 0x80200000u) <= 0x00400000u || !(fabsf(t) <= 64.0f);
-  return h;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(t0));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(t1));
+  unpack_f32x2(add_f32x2(f32x2(e0, e1), one), d0, d1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(d1));
+  unpack_f32x2(mul_f32x2(u, mul_f32x2(g, f32x2(r0, r1))), h0, h1);
+  t_abs = fmaxf(fabsf(t0), fabsf(t1));
 }
 
 // two floats -> packed bf16x2 (round to nearest even), lo in the low half

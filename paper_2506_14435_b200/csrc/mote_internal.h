@@ -22,7 +22,7 @@ struct QuantActArgs {
   const int32_t* topk_idx; const int32_t* blk_base; int E; int n_blk;
   // few blocks (n_blk <= kInlineScanBlocks, blk_base null): every CTA derives the bases from the router's block counts,
   // and the first one writes the tables that launch_dispatch_scan would have written
-  const int32_t* blk_hist; int32_t* offsets_out; int4* tiles_routed; int4* tiles_shared;
+  const int32_t* blk_hist; int32_t* offsets_out; int4* tiles_routed; int4* tiles_shared; int cg_routed, cg_shared;
   int32_t* perm_out; int32_t* inv_out;
   uint32_t* zero_u32; int32_t* zero_i32;   // optional [rows] arrays cleared at every destination row
   int k;
@@ -54,9 +54,11 @@ mote_status_t launch_dispatch(const int32_t* idx, int64_t P, int E, int32_t* off
                               int32_t* inv, int4* tiles_routed, int4* tiles_shared, int64_t T,
                               cudaStream_t stream);
 
-// Block-wise variant: offsets, per-block bases and the tile tables from the router's block histograms.
+// Block-wise variant: offsets, per-block bases and the tile tables (of 128 * cg rows per tile) from the router's block
+// histograms.
 mote_status_t launch_dispatch_scan(const int32_t* blk_hist, int n_blk, int E, int32_t* offsets, int32_t* blk_base,
-                                   int4* tiles_routed, int4* tiles_shared, int64_t T, cudaStream_t stream);
+                                   int4* tiles_routed, int cg_routed, int4* tiles_shared, int cg_shared, int64_t T,
+                                   cudaStream_t stream);
 
 // CUDA-core (dp4a) grouped ternary GEMMs.  qa rows are in expert-sorted order, canonical k order.
 struct TernaryGemmArgs {
@@ -80,10 +82,11 @@ mote_status_t launch_ternary_down_simt(const TernaryGemmArgs& a, cudaStream_t st
 
 // Tensor-core (tcgen05) versions.  qa must be stored k-interleaved (see quant_act.cu); needs
 // K % 128 == 0 and N % 128 == 0.
+// cg: CTAs per tile, 1 or 2; `tiles` holds row tiles of 128 * cg rows.
 // beta_out_bits (gate/up only, may be null): per row, atomicMax of the bits of |h| (must be zeroed).
 mote_status_t launch_ternary_umma(const TernaryGemmArgs& a, bool gateup, const int4* tiles, int max_mtiles,
                                   const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status,
-                                  cudaStream_t stream, bool pdl = false);
+                                  cudaStream_t stream, bool pdl = false, int cg = 1);
 
 // Q_a(h) for rows whose absmax is already known: beta_bits holds max |h| per row (raw bits);
 // writes q (k-interleaved if asked), the clamped beta in place, and accumulates rowsum (zeroed).
@@ -101,12 +104,13 @@ struct SharedMat { const void* w; const float* scale; };
 struct CombineArgs {
   const float* y; const float* w; const int32_t* perm; const void* residual; void* out; int k;
 };
+// cg = 2: bf16 operands only.
 // k_splits > 1 (down projection only, no comb): `out` receives k_splits partial outputs of T x N
 // floats each, to be added in ascending order (see shared_down_k_splits).
 mote_status_t launch_shared_umma(const void* act, const SharedMat& w0, const SharedMat& w1, int bits, bool gateup,
                                  int64_t T, int K, int N, void* out, const int4* tiles, int max_mtiles,
                                  uint32_t* status, const CombineArgs* comb, cudaStream_t stream, bool pdl = false,
-                                 int k_splits = 1);
+                                 int k_splits = 1, int cg = 1);
 // The routed GEMM and the shared expert's GEMM of the same step (gate/up, or down) as one launch; `act`, w0, w1, bits, T,
 // out, tiles_shared, k_splits: the shared one's, as in launch_shared_umma.
 mote_status_t launch_umma_pair(const TernaryGemmArgs& g, bool gateup, const int4* tiles_routed, int max_mtiles_routed,
@@ -118,6 +122,9 @@ mote_status_t launch_umma_pair(const TernaryGemmArgs& g, bool gateup, const int4
 mote_status_t launch_bounded_wait_selftest(uint32_t* status, uint64_t limit_ns, cudaStream_t stream);
 constexpr int64_t kMaxPartialRows = 4096;
 int shared_down_k_splits(int64_t T, int N, int K);
+// CTAs per tile (1 or 2) of the routed experts' and of the shared expert's two GEMMs where each is a launch of its own.
+int routed_ctas_per_tile(int64_t P, int E, int d, int f);
+int shared_ctas_per_tile(int64_t T, int d, int f, int k_splits);
 
 // CUDA-core GEMMs of the shared expert.
 mote_status_t launch_shared_gateup_simt(const void* x, const SharedMat& Wg, const SharedMat& Wu, int bits, int64_t T,

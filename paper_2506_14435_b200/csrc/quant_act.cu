@@ -44,7 +44,7 @@ __device__ __forceinline__ void scan_block_counts(const QuantActArgs& a, InlineS
   __syncthreads();
   if (warp == 0) {
     const int c0 = lane < E ? sc.count[lane] : 0, c1 = lane + 32 < E ? sc.count[lane + 32] : 0;
-    const int n0 = (c0 + 127) / 128, n1 = (c1 + 127) / 128;
+    const int tr = 128 * a.cg_routed, n0 = (c0 + tr - 1) / tr, n1 = (c1 + tr - 1) / tr;
     const int r0 = scan_inclusive(c0, lane), t0 = scan_inclusive(n0, lane);
     const int r1 = scan_inclusive(c1, lane) + __shfl_sync(0xffffffffu, r0, 31);
     const int t1 = scan_inclusive(n1, lane) + __shfl_sync(0xffffffffu, t0, 31);
@@ -52,14 +52,14 @@ __device__ __forceinline__ void scan_block_counts(const QuantActArgs& a, InlineS
     if (blockIdx.x == 0) {
       if (lane < E) a.offsets_out[lane] = r0 - c0;
       if (lane + 32 < E) a.offsets_out[lane + 32] = r1 - c1;
-      for (int i = 0; i < n0; ++i) a.tiles_routed[1 + t0 - n0 + i] = make_int4(lane, r0 - c0 + 128 * i, min(128, c0 - 128 * i), 0);
-      for (int i = 0; i < n1; ++i) a.tiles_routed[1 + t1 - n1 + i] = make_int4(lane + 32, r1 - c1 + 128 * i, min(128, c1 - 128 * i), 0);
+      for (int i = 0; i < n0; ++i) a.tiles_routed[1 + t0 - n0 + i] = make_int4(lane, r0 - c0 + tr * i, min(tr, c0 - tr * i), 0);
+      for (int i = 0; i < n1; ++i) a.tiles_routed[1 + t1 - n1 + i] = make_int4(lane + 32, r1 - c1 + tr * i, min(tr, c1 - tr * i), 0);
       if (lane == 31) {
         a.offsets_out[E] = r1;
         a.tiles_routed[0] = make_int4(t1, 0, 0, 0);
       }
-      const int T = (int)a.T, n = (T + 127) / 128;
-      for (int i = lane; i < n; i += 32) a.tiles_shared[1 + i] = make_int4(0, i * 128, min(128, T - i * 128), 0);
+      const int T = (int)a.T, ts = 128 * a.cg_shared, n = (T + ts - 1) / ts;
+      for (int i = lane; i < n; i += 32) a.tiles_shared[1 + i] = make_int4(0, i * ts, min(ts, T - i * ts), 0);
       if (lane == 0) a.tiles_shared[0] = make_int4(n, 0, 0, 0);
     }
   }

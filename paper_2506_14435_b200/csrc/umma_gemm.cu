@@ -29,11 +29,19 @@
 // 1 TMA producer of packed weights, 2 MMA issuer + TMEM owner, 4-11 two groups of unpackers
 // that take alternate pipeline stages, 12-19 epilogue (two warps per TMEM lane quarter, each
 // owning half of the tile's columns).
+// Pairs of CTAs (CG = 2, clusters of two; long prefills, see routed_ctas_per_tile): a tile is 256 token rows, 128 in either
+// CTA, and cta_group::2 MMAs, issued by the first CTA, read half of the weight rows from each.  So either CTA fetches, expands and
+// keeps 128 weight rows instead of 256 for the same MMA work (32 KB per stage instead of 48, six stages instead of three), and an
+// SM's shared memory moves 72 KB per step instead of 112 in the 512 cycles that the step's MMAs take.  The second CTA's copies and
+// announcements go to the first one's `full` barriers; commits arrive at both.  2048 x 11008, 8192 tokens, 16 experts: routed
+// gate/up 595 -> 435 us (3 400 TOP/s), routed down 300 -> 224.  Half of that is the issue loop (see issue_mmas).
+//
 // Two accumulator buffers of 256 TMEM columns let the epilogue of one tile overlap the MMAs of
 // the next.  Every mbarrier wait is bounded; on expiry the CTA raises a status word and leaves.
 #include <cuda.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "mote_common.cuh"
@@ -51,7 +59,9 @@ constexpr int kBM = 128;
 constexpr int kStageA = kBM * 128;             // 16 KB: 128 rows x 128 B
 constexpr int kStageB = 256 * 128;             // 32 KB: up to 256 rows x 128 B
 constexpr int kStagesTernary = 3, kStagesBf16 = 4, kStagesRtn = 3;
-constexpr int kThreads = 640;
+constexpr int kStagesPaired = 6;               // half the weight rows per CTA: 32 KB per stage
+constexpr int kMaxStages = 6;
+constexpr int kFirstEpilogueWarp = 12;
 constexpr int kTmemCols = 512;
 
 struct UmmaArgs {
@@ -81,28 +91,32 @@ struct UmmaArgs {
 };
 
 struct __align__(8) PipeBarriers {
-  uint64_t full_a[4], empty[4], full_u[4], full_p[4], empty_p[4], tmem_full[2], tmem_empty[2];
+  uint64_t full[kMaxStages], empty[kMaxStages], full_p[kMaxStages], empty_p[kMaxStages], tmem_full[2], tmem_empty[2];
   uint32_t tmem_base;
   int abort_flag;
 };
 
-template <int MODE>
+// CG: CTAs per tile (see the head of this file)
+template <int MODE, int CG = 1>
 struct ModeTraits {
   static constexpr bool kTernary = (MODE == MODE_T_GATEUP || MODE == MODE_T_DOWN);
   static constexpr int kRtnBits = MODE >= MODE_Q4_GATEUP ? 4 : MODE >= MODE_Q8_GATEUP ? 8 : 0;
   static constexpr bool kRtn = kRtnBits != 0;
   static constexpr bool kUnpack = kTernary || kRtn;       // weights reach shared memory as codes
   static constexpr bool kGateUp = (MODE % 2 == 0);
-  static constexpr int kStages = kTernary ? kStagesTernary : kRtn ? kStagesRtn : kStagesBf16;
+  static constexpr int kStageB = mote::kStageB / CG;
+  static constexpr int kStages = CG == 2 ? kStagesPaired : kTernary ? kStagesTernary : kRtn ? kStagesRtn : kStagesBf16;
   // code bytes per weight row and pipeline stage: 128 2-bit codes, 64 int8 codes or 64 4-bit codes
   static constexpr int kCodeRowBytes = kRtnBits == 8 ? 64 : 32;
-  static constexpr int kStageP = 256 * kCodeRowBytes;     // up to 256 rows
-  static constexpr int kStagesP = kRtnBits == 8 ? 3 : 4;
+  static constexpr int kStageP = 256 * kCodeRowBytes / CG;     // up to 256 rows, half of them per CTA of a pair
+  static constexpr int kStagesP = CG == 2 ? kStagesPaired : kRtnBits == 8 ? 3 : 4;
   // gate/up epilogue: every epilogue warp stages 32 rows x kEpiCols bf16 (row pitch padded by 16 B)
   // and writes them out as whole row segments
   // (bf16 gate/up only.  For the ternary gate/up, whose epilogue competes with the unpackers for
   // issue slots, staging -- with plain stores or with a TMA store -- measured slower than letting
   // every thread write its own 32 bytes.)
+  static constexpr int kEpiWarps = 8;
+  static constexpr int kThreads = (kFirstEpilogueWarp + kEpiWarps) * 32;
   static constexpr int kEpiCols = 32;
   static constexpr int kEpiPitch = kEpiCols * 2 + 16;
   static constexpr size_t kEpiStage = (kGateUp && !kTernary) ? size_t(8) * 32 * kEpiPitch : 0;
@@ -111,18 +125,21 @@ struct ModeTraits {
 };
 
 // What a CTA of one GEMM (SMODE < 0) or of a pair of GEMMs lays out in shared memory.
-template <int MODE, int SMODE>
+template <int MODE, int SMODE, int CG>
 struct PairTraits {
+  static_assert(CG == 1, "pairs of GEMMs run on single CTAs");
+  static constexpr int kStageB = mote::kStageB;
   using TR = ModeTraits<MODE>; using TS = ModeTraits<SMODE>;
   static constexpr bool kGateUp = TR::kGateUp, kUnpack = true;
+  static constexpr int kEpiWarps = TR::kEpiWarps, kThreads = TR::kThreads;
   static constexpr int kStages = kStagesTernary;
   static constexpr int kStageP = std::max(TR::kStageP, TS::kUnpack ? TS::kStageP : 0);
   static constexpr int kStagesP = TS::kRtnBits == 8 ? 3 : 4;
   static constexpr size_t kEpiStage = TS::kEpiStage;
   static constexpr size_t kSmem = 1024 + size_t(kStages) * (kStageA + kStageB) + size_t(kStagesP) * kStageP + kEpiStage + sizeof(PipeBarriers);
 };
-template <int MODE>
-struct PairTraits<MODE, -1> : ModeTraits<MODE> {};
+template <int MODE, int CG>
+struct PairTraits<MODE, -1, CG> : ModeTraits<MODE, CG> {};
 
 // Item order.  The CTAs of the grid work on neighbouring items at the same time, and the operand
 // those items share is the one L2 serves to all of them from a single HBM read.
@@ -145,12 +162,12 @@ struct PairTraits<MODE, -1> : ModeTraits<MODE> {};
 // 332 / 312; 2048 x 5632 203 / 192; INT8, 4 experts, 384 tokens 160 / 158).
 struct ItemPlan { int n_items, n_whole; };
 template <bool kGateUp>
-__device__ __forceinline__ ItemPlan plan_items(const UmmaArgs& a, int n_mtiles) {
+__device__ __forceinline__ ItemPlan plan_items(const UmmaArgs& a, int n_mtiles, int workers) {
   ItemPlan p;
   p.n_items = p.n_whole = n_mtiles * a.n_ntiles * (kGateUp ? 1 : a.k_splits);
   if (!kGateUp && a.split_tail) {
-    const int tail = p.n_items % (int)gridDim.x;
-    if (tail > 0 && 2 * tail <= (int)gridDim.x) { p.n_whole = p.n_items - tail; p.n_items += tail; }
+    const int tail = p.n_items % workers;
+    if (tail > 0 && 2 * tail <= workers) { p.n_whole = p.n_items - tail; p.n_items += tail; }
   }
   return p;
 }
@@ -211,50 +228,64 @@ struct RingPos {
   }
 };
 
-// the token operand, and the weights where they are bf16
-template <int MODE, int S>
+// The weight rows of one stage that this CTA fetches.  One CTA per tile: gate rows and up rows, or the (up to) 256 rows of a
+// down tile, as two boxes.  A pair: the first CTA the gate rows and the second the up rows, or either half of a down tile; there
+// the box is half a tile, or 64 rows where a tile is 256 wide, since it may be cut into halves (weight_box_rows).
+template <int MODE, int CG, typename Load>
+__device__ __forceinline__ void load_weight_rows(const CUtensorMap& tm_b0, const CUtensorMap& tm_b1, const UmmaArgs& a, uint32_t dst,
+                                                 int row_bytes, int b_row, int width, uint32_t rank, Load&& load) {
+  using TR = ModeTraits<MODE, CG>;
+  if (CG == 1) {
+    load(dst, tm_b0, b_row);
+    if (TR::kGateUp) load(dst + 128 * row_bytes, tm_b1, b_row);
+    else if (width > 128) load(dst + 128 * row_bytes, tm_b1, b_row + 128);
+  } else if (TR::kGateUp) {
+    load(dst, rank ? tm_b1 : tm_b0, b_row);
+  } else {
+    b_row += (int)rank * (width / 2);
+    load(dst, tm_b0, b_row);
+    if (a.bn == 256 && width > 128) load(dst + 64 * row_bytes, tm_b0, b_row + 64);
+  }
+}
+
+// the token operand, and the weights where they are bf16.  In a pair either CTA fetches its own 128 token rows and its half
+// of the weight rows; all of it is counted on the first CTA's barrier, where the MMA issuer waits.
+template <int MODE, int S, int CG>
 __device__ __forceinline__ bool load_operands(const CUtensorMap& tm_a, const CUtensorMap& tm_b0, const CUtensorMap& tm_b1,
                                               const UmmaArgs& a, int item, int n_mtiles, int n_whole, uint32_t sA, uint32_t sB,
-                                              PipeBarriers* bars, RingPos& p) {
-  using TR = ModeTraits<MODE>;
+                                              PipeBarriers* bars, uint32_t rank, RingPos& p) {
+  using TR = ModeTraits<MODE, CG>;
   volatile int* abort_flag = &bars->abort_flag;
   int4 tile; int n_tile, half;
   decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
   const int width = half < 0 ? a.bn : 128;
   const int b_row = (a.b_rows_per_expert ? tile.x * a.b_rows_per_expert : 0) +
                     n_tile * (TR::kGateUp ? a.bn / 2 : a.bn) + (half > 0 ? 128 : 0);
+  const int a_row = tile.y + (int)rank * kBM;
+  constexpr int kCols = TR::kTernary ? 128 : 64;           // elements in the 128 bytes of a stage's row
   int kb, ke;
   item_k_range<TR::kGateUp>(a, item, kb, ke);
   for (int ks = kb; ks < ke; ++ks) {
     if (!mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, abort_flag)) return false;
-    const uint32_t bar = smem_u32(&bars->full_a[p.stage]);
-    if (TR::kTernary) {
-      mbar_expect_tx(bar, kStageA);
-      tma_load_2d(sA + p.stage * kStageA, &tm_a, ks * 128, tile.y, bar);
-    } else if (TR::kRtn) {
-      mbar_expect_tx(bar, kStageA);
-      tma_load_2d(sA + p.stage * kStageA, &tm_a, ks * 64, tile.y, bar);
-    } else {
-      mbar_expect_tx(bar, kStageA + width * 128);
-      tma_load_2d(sA + p.stage * kStageA, &tm_a, ks * 64, tile.y, bar);
-      if (TR::kGateUp) {
-        tma_load_2d(sB + p.stage * kStageB, &tm_b0, ks * 64, b_row, bar);
-        tma_load_2d(sB + p.stage * kStageB + 128 * 128, &tm_b1, ks * 64, b_row, bar);
-      } else {
-        tma_load_2d(sB + p.stage * kStageB, &tm_b0, ks * 64, b_row, bar);
-        if (width > 128) tma_load_2d(sB + p.stage * kStageB + 128 * 128, &tm_b1, ks * 64, b_row + 128, bar);
-      }
-    }
+    uint32_t bar = smem_u32(&bars->full[p.stage]);
+    if (CG == 1 || rank == 0) mbar_expect_tx(bar, CG * kStageA + (TR::kUnpack ? 0 : width * 128));
+    if (CG == 2) bar = map_to_rank(bar, 0);
+    auto load = [&](uint32_t dst, const CUtensorMap& tm, int row) {
+      if (CG == 2) tma_load_2d_pair(dst, &tm, ks * kCols, row, bar);
+      else tma_load_2d(dst, &tm, ks * kCols, row, bar);
+    };
+    load(sA + p.stage * kStageA, tm_a, a_row);
+    if (!TR::kUnpack) load_weight_rows<MODE, CG>(tm_b0, tm_b1, a, sB + p.stage * TR::kStageB, 128, b_row, width, rank, load);
     p.next(S);
   }
   return true;
 }
 
-// weight codes
-template <int MODE, int kStagesP, int kStageP>
+// weight codes (a pair: either CTA the codes of its half of the weight rows, on its own barrier)
+template <int MODE, int kStagesP, int kStageP, int CG>
 __device__ __forceinline__ bool load_codes(const CUtensorMap& tm_b0, const CUtensorMap& tm_b1, const UmmaArgs& a, int item, int n_mtiles, int n_whole,
-                                           uint32_t sP, PipeBarriers* bars, RingPos& p) {
-  using TR = ModeTraits<MODE>;
+                                           uint32_t sP, PipeBarriers* bars, uint32_t rank, RingPos& p) {
+  using TR = ModeTraits<MODE, CG>;
   volatile int* abort_flag = &bars->abort_flag;
   constexpr int kRB = TR::kCodeRowBytes;
   int4 tile; int n_tile, half;
@@ -266,63 +297,65 @@ __device__ __forceinline__ bool load_codes(const CUtensorMap& tm_b0, const CUten
   for (int ks = kb; ks < ke; ++ks) {
     if (!mbar_wait(smem_u32(&bars->empty_p[p.stage]), p.phase ^ 1, abort_flag)) return false;
     const uint32_t bar = smem_u32(&bars->full_p[p.stage]);
-    mbar_expect_tx(bar, width * kRB);
-    const uint32_t dst = sP + p.stage * kStageP;
-    if (TR::kGateUp) {
-      tma_load_2d(dst, &tm_b0, ks * kRB, b_row, bar);
-      tma_load_2d(dst + 128 * kRB, &tm_b1, ks * kRB, b_row, bar);
-    } else {
-      tma_load_2d(dst, &tm_b0, ks * kRB, b_row, bar);
-      if (width > 128) tma_load_2d(dst + 128 * kRB, &tm_b1, ks * kRB, b_row + 128, bar);
-    }
+    mbar_expect_tx(bar, width / CG * kRB);
+    load_weight_rows<MODE, CG>(tm_b0, tm_b1, a, sP + p.stage * kStageP, kRB, b_row, width, rank,
+                               [&](uint32_t dst, const CUtensorMap& tm, int row) { tma_load_2d(dst, &tm, ks * kRB, row, bar); });
     p.next(kStagesP);
   }
   return true;
 }
 
-// kWaitU: the unpackers announce every pipeline stage
-template <int MODE, int S, bool kWaitU>
+// A whole warp walks the steps (in a pair the first CTA's, for both) and one elected lane issues.  Warp-uniform control flow is
+// what keeps descriptors and barrier addresses in uniform registers, where tcgen05.mma takes its operands: with one lane in a
+// loop of its own a step of four MMAs took the issuing thread 830 to 870 cycles beside busy unpackers and epilogue warps, and
+// the tensor pipe, which needs 512, waited for it.
+template <int MODE, int S, int CG>
 __device__ __forceinline__ bool issue_mmas(const UmmaArgs& a, int item, int n_whole, int local, uint32_t tmem_base, uint32_t sA,
                                            uint32_t sB, PipeBarriers* bars, RingPos& p) {
-  using TR = ModeTraits<MODE>;
+  using TR = ModeTraits<MODE, CG>;
   volatile int* abort_flag = &bars->abort_flag;
-  const uint32_t idesc_whole = TR::kTernary ? make_idesc(2, 1, 0, kBM, (uint32_t)a.bn)     // s32 += s8 * u8
-                                            : make_idesc(1, 1, 1, kBM, (uint32_t)a.bn);    // f32 += bf16 * bf16
-  const uint32_t idesc_half = TR::kTernary ? make_idesc(2, 1, 0, kBM, 128u) : make_idesc(1, 1, 1, kBM, 128u);
+  constexpr uint32_t kM = kBM * CG;
+  const uint32_t idesc_whole = TR::kTernary ? make_idesc(2, 1, 0, kM, (uint32_t)a.bn)     // s32 += s8 * u8
+                                            : make_idesc(1, 1, 1, kM, (uint32_t)a.bn);    // f32 += bf16 * bf16
+  const uint32_t idesc_half = TR::kTernary ? make_idesc(2, 1, 0, kM, 128u) : make_idesc(1, 1, 1, kM, 128u);
   const int buf = local & 1;
   const uint32_t use = (uint32_t)(local >> 1);
-  if (!mbar_wait(smem_u32(&bars->tmem_empty[buf]), (use & 1) ^ 1, abort_flag)) return false;
+  if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->tmem_empty[buf]), (use & 1) ^ 1, abort_flag))) return false;
   tc_fence_after();
   const uint32_t d_tmem = tmem_base + buf * 256;
   const uint32_t idesc = (!TR::kGateUp && item >= n_whole) ? idesc_half : idesc_whole;
   int kb, ke;
   item_k_range<TR::kGateUp>(a, item, kb, ke);
+  uint32_t acc = 0;
   for (int ks = kb; ks < ke; ++ks) {
-    if (!mbar_wait(smem_u32(&bars->full_a[p.stage]), p.phase, abort_flag)) return false;
-    if (kWaitU)
-      if (!mbar_wait(smem_u32(&bars->full_u[p.stage]), p.phase, abort_flag)) return false;
+    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->full[p.stage]), p.phase, abort_flag))) return false;
     tc_fence_after();
     const uint64_t da = smem_desc_sw128(sA + p.stage * kStageA);
-    const uint64_t db = smem_desc_sw128(sB + p.stage * kStageB);
+    const uint64_t db = smem_desc_sw128(sB + p.stage * TR::kStageB);
+    if (elect_one()) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t acc = (ks > kb || j > 0) ? 1u : 0u;
-      if (TR::kTernary) mma_i8(d_tmem, da + 2 * j, db + 2 * j, idesc, acc);
-      else mma_f16(d_tmem, da + 2 * j, db + 2 * j, idesc, acc);
+      for (int j = 0; j < 4; ++j) {
+        if (TR::kTernary) mma_i8<CG>(d_tmem, da + 2 * j, db + 2 * j, idesc, j > 0 ? 1u : acc);
+        else mma_f16<CG>(d_tmem, da + 2 * j, db + 2 * j, idesc, j > 0 ? 1u : acc);
+      }
+      mma_commit<CG>(smem_u32(&bars->empty[p.stage]));
     }
-    mma_commit(smem_u32(&bars->empty[p.stage]));
+    __syncwarp();
+    acc = 1;
     p.next(S);
   }
-  mma_commit(smem_u32(&bars->tmem_full[buf]));
+  if (elect_one()) mma_commit<CG>(smem_u32(&bars->tmem_full[buf]));
+  __syncwarp();
   return true;
 }
 
 // 2-bit -> int8 for the ternary experts; int8 / 4-bit -> bf16 for an RTN-coded shared expert.  group 0 (warps 4-7)
 // expands the even pipeline steps, group 1 (warps 8-11) the odd ones.  p, q: positions in the rings of stages and codes
-template <int MODE, int S, int kStagesP, int kStageP>
+// (a pair: either CTA its half of the rows; the MMA issuer, in the first CTA, is told by both)
+template <int MODE, int S, int kStagesP, int kStageP, int CG>
 __device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_whole, int group, uint8_t* genB,
                                              const uint8_t* genP, PipeBarriers* bars, RingPos& p, RingPos& q, uint32_t& step) {
-  using TR = ModeTraits<MODE>;
+  using TR = ModeTraits<MODE, CG>;
   volatile int* abort_flag = &bars->abort_flag;
   const int tid = (threadIdx.x - 128) & 127, lane = threadIdx.x & 31;
   if constexpr (!TR::kUnpack) {                    // bf16 weights among items with codes: only the announcements
@@ -331,12 +364,12 @@ __device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_
     for (int ks = kb; ks < ke; ++ks, ++step, p.next(S)) {
       if ((step & 1u) != (uint32_t)group) continue;
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, abort_flag))) return false;
-      if (lane == 0) mbar_arrive(smem_u32(&bars->full_u[p.stage]));
+      if (lane == 0) mbar_arrive(smem_u32(&bars->full[p.stage]));
     }
     return true;
   }
   // chunks of 16 code bytes, spread over 128 threads
-  const int n_chunks = ((!TR::kGateUp && item >= n_whole) ? 128 : a.bn) * (TR::kCodeRowBytes / 16);
+  const int n_chunks = ((!TR::kGateUp && item >= n_whole) ? 128 : a.bn) / CG * (TR::kCodeRowBytes / 16);
   int kb, ke;
   item_k_range<TR::kGateUp>(a, item, kb, ke);
   for (int ks = kb; ks < ke; ++ks, ++step) {
@@ -350,7 +383,7 @@ __device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_
                       mbar_wait(smem_u32(&bars->full_p[q.stage]), q.phase, abort_flag);
       if (!__all_sync(0xffffffffu, ok)) return false;
       const uint8_t* src = genP + q.stage * kStageP;
-      uint8_t* dst = genB + p.stage * kStageB;
+      uint8_t* dst = genB + p.stage * TR::kStageB;
       // batches of four chunks per thread, all loads of a batch ahead of its conversions
       for (int c0 = tid; c0 < n_chunks; c0 += 128 * 4) {
         uint4 wv[4];
@@ -398,7 +431,8 @@ __device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_
       fence_proxy_async_smem();                // generic-proxy writes -> visible to the MMA
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(smem_u32(&bars->full_u[p.stage]));
+        if (CG == 2) mbar_arrive_cluster(map_to_rank(smem_u32(&bars->full[p.stage]), 0));
+        else mbar_arrive(smem_u32(&bars->full[p.stage]));
         mbar_arrive(smem_u32(&bars->empty_p[q.stage]));
       }
     }
@@ -408,24 +442,26 @@ __device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_
   return true;
 }
 
-template <int MODE>
+template <int MODE, int CG>
 __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mtiles, int n_whole, int local, uint32_t tmem_base,
-                                          uint8_t* genE, PipeBarriers* bars) {
-  using TR = ModeTraits<MODE>;
+                                          uint8_t* genE, PipeBarriers* bars, uint32_t rank) {
+  using TR = ModeTraits<MODE, CG>;
   volatile int* abort_flag = &bars->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;                          // TMEM lane quarter this warp may read
-  const int chalf = (warp - 12) >> 2;              // which half of the tile's columns
+  constexpr int kParts = TR::kEpiWarps / 4;         // warps per lane quarter
+  const int part = (warp - kFirstEpilogueWarp) >> 2;   // which part of the tile's columns
   const int r_in_tile = q * 32 + lane;
   int4 tile; int n_tile, half;
   decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
+  if (CG == 2) {                                   // this CTA's 128 rows of the pair's tile
+    tile.y += (int)rank * kBM;
+    tile.z = min(tile.z - (int)rank * kBM, kBM);
+  }
   int kb_, ke_;
   const int split = item_k_range<TR::kGateUp>(a, item, kb_, ke_);
   const int buf = local & 1;
   const uint32_t use = (uint32_t)(local >> 1);
-  const bool ok = mbar_wait(smem_u32(&bars->tmem_full[buf]), use & 1, abort_flag);
-  if (!__all_sync(0xffffffffu, ok)) return false;
-  tc_fence_after();
   const bool row_ok = r_in_tile < tile.z;
   const int64_t row = int64_t(tile.y) + r_in_tile;
   const uint32_t t_row = tmem_base + (uint32_t(q * 32) << 16) + buf * 256;
@@ -437,16 +473,20 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
     c0 = dequant_scale(a.alpha0[tile.x], beta);
     if (TR::kGateUp) c1 = dequant_scale(a.alpha1[tile.x], beta);
   }
+  const bool ok = mbar_wait(smem_u32(&bars->tmem_full[buf]), use & 1, abort_flag);
+  if (!__all_sync(0xffffffffu, ok)) return false;
+  tc_fence_after();
   if (TR::kGateUp) {
     const int col0 = n_tile * 128;
     const bool row_fast = __fmul_rn(c0, c1) > 1e-12f;
     const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;
+    const uint64_t c0x2 = f32x2(c0, c0), c1x2 = f32x2(c1, c1);
     float hmax = 0.0f;                           // max |h| (before the bf16 rounding, which is monotonic)
     constexpr int kCols = TR::kEpiCols, kPitch = TR::kEpiPitch;
     constexpr int kLanesPerRow = kCols * 2 / 16, kRowsPerStore = 32 / kLanesPerRow;
-    uint8_t* stg = genE + (warp - 12) * 32 * kPitch;
+    uint8_t* stg = genE + (warp - kFirstEpilogueWarp) * 32 * kPitch;
 #pragma unroll 1
-    for (int cr = chalf * 64; cr < chalf * 64 + 64; cr += kCols) {
+    for (int cr = part * (128 / kParts); cr < (part + 1) * (128 / kParts); cr += kCols) {
 #pragma unroll 1
       for (int c = cr; c < cr + kCols; c += 16) {
         uint32_t rg[16], ru[16];
@@ -456,25 +496,24 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
         if (row_ok) {
           float hv[16];
           if (TR::kTernary) {
-            uint32_t redo_mask = 0u;
+            float t_max = row_fast ? 0.0f : INFINITY;
+            uint32_t key = 0xFFFFFFFFu;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              bool redo;
-              hv[j] = glu_h_fast_biased(rg[j], ru[j], acc_bias, c0, c1, redo);
-              if (redo) redo_mask |= 1u << j;
+            for (int j = 0; j < 16; j += 2) {
+              float t;
+              glu_h2_fast_biased(rg[j], rg[j + 1], ru[j], ru[j + 1], acc_bias, c0x2, c1x2, hv[j], hv[j + 1], t);
+              t_max = fmaxf(t_max, t);
+              key = min(key, min(glu_midpoint_key(hv[j]), glu_midpoint_key(hv[j + 1])));
             }
-            if (!row_fast) redo_mask = 0xFFFFu;
-            if (redo_mask) {                     // mostly one element: look at four at a time
+            const bool all = !(t_max <= kGluMaxT);
+            if (key <= kGluMidpointKeys || all) {        // mostly one element
 #pragma unroll
-              for (int j0 = 0; j0 < 16; j0 += 4)
-                if ((redo_mask >> j0) & 0xFu) {
-#pragma unroll
-                  for (int j = j0; j < j0 + 4; ++j)
-                    if ((redo_mask >> j) & 1u) hv[j] = glu_h_rare((int)rg[j] - rs, (int)ru[j] - rs, c0, c1);
-                }
+              for (int j = 0; j < 16; ++j)
+                if (glu_midpoint_key(hv[j]) <= kGluMidpointKeys || all)
+                  hv[j] = glu_h_rare((int)rg[j] - rs, (int)ru[j] - rs, c0, c1);
             }
 #pragma unroll
-            for (int j = 0; j < 16; ++j) hmax = fmaxf(hmax, fabsf(hv[j]));
+            for (int j = 0; j < 16; j += 2) hmax = fmaxf(fmaxf(hmax, fabsf(hv[j])), fabsf(hv[j + 1]));
           } else if (TR::kRtn || a.alpha0 != nullptr) {
             // RTN-coded shared expert (codes expanded here, or beforehand): row scales of the
             // gate and up matrices = scales of this tile's output columns
@@ -541,10 +580,10 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
       if (hb) atomicMax(a.beta_out_bits + row, hb);
     }
   } else {
-    const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;   // see glu_h_fast_biased
+    const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;   // see glu_h2_fast_biased
     const int width = half < 0 ? a.bn : 128;
     const int col0 = n_tile * a.bn + (half > 0 ? 128 : 0);
-    const int cbeg = chalf * (width / 2), cend = cbeg + width / 2;
+    const int cbeg = part * (width / kParts), cend = cbeg + width / kParts;
     const bool combine = !TR::kTernary && a.comb_out != nullptr;
     float cw[MOTE_MAX_TOPK];
     const float* cy[MOTE_MAX_TOPK];
@@ -630,7 +669,10 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
   }
   tc_fence_before();
   __syncwarp();
-  if (lane == 0) mbar_arrive(smem_u32(&bars->tmem_empty[buf]));
+  if (lane == 0) {
+    if (CG == 2) mbar_arrive_cluster(map_to_rank(smem_u32(&bars->tmem_empty[buf]), 0));
+    else mbar_arrive(smem_u32(&bars->tmem_empty[buf]));
+  }
   return true;
 }
 
@@ -638,10 +680,10 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
 // The CTA's walk over its items: all of mode MODE, or (pair of GEMMs) routed items of mode MODE and shared items of
 // mode SMODE.  A pair takes the longer items first: gate/up the shared ones (bf16 rows are eight times as long as 2-bit
 // ones), down the routed ones (the shared ones are cut along K).
-template <int MODE, int SMODE>
+template <int MODE, int SMODE, int CG>
 __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensorMap& tm_b0, const CUtensorMap& tm_b1, const UmmaArgs& a,
                                          const CUtensorMap& ts_a, const CUtensorMap& ts_b0, const CUtensorMap& ts_b1, const UmmaArgs& as) {
-  using TR = PairTraits<MODE, SMODE>;
+  using TR = PairTraits<MODE, SMODE, CG>;
   constexpr bool kPair = SMODE >= 0;
   constexpr int kS = kPair ? SMODE : MODE;
   constexpr int S = TR::kStages, kStagesP = TR::kStagesP, kStageP = TR::kStageP;
@@ -650,26 +692,28 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
   const uint32_t sA = smem_base;
   const uint32_t sB = sA + S * kStageA;
-  const uint32_t sP = sB + S * kStageB;
+  const uint32_t sP = sB + S * TR::kStageB;
   uint8_t* genB = smem_gen + S * kStageA;
-  uint8_t* genP = genB + S * kStageB;
+  uint8_t* genP = genB + S * TR::kStageB;
   uint8_t* genE = genP + (TR::kUnpack ? kStagesP * kStageP : 0);
   PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(genE + TR::kEpiStage);
   volatile int* abort_flag = &bars->abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const uint32_t rank = CG == 2 ? cluster_ctarank() : 0;
+  const int worker = blockIdx.x / CG, workers = gridDim.x / CG;      // CTAs, or pairs of them
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 4; ++s) {
-      mbar_init(smem_u32(&bars->full_a[s]), 1);
+    for (int s = 0; s < kMaxStages; ++s) {
+      // the operands have landed, and four unpacking warps per CTA have announced their part
+      mbar_init(smem_u32(&bars->full[s]), 1 + (TR::kUnpack ? 4 * CG : 0));
       mbar_init(smem_u32(&bars->empty[s]), 1);
-      mbar_init(smem_u32(&bars->full_u[s]), 4);
       mbar_init(smem_u32(&bars->full_p[s]), 1);
       mbar_init(smem_u32(&bars->empty_p[s]), 4);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars->tmem_full[b]), 1);
-      mbar_init(smem_u32(&bars->tmem_empty[b]), 8);
+      mbar_init(smem_u32(&bars->tmem_empty[b]), TR::kEpiWarps * CG);
     }
     bars->abort_flag = 0;
     fence_barrier_init();
@@ -683,20 +727,21 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
     }
   }
   if (warp == 2) {
-    tmem_alloc(smem_u32(&bars->tmem_base), kTmemCols);
-    tmem_relinquish();
+    tmem_alloc<CG>(smem_u32(&bars->tmem_base), kTmemCols);
+    tmem_relinquish<CG>();
   }
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync();             // the other CTA's barriers are initialised
   tc_fence_after();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   pdl_wait();                              // set-up above overlaps the tail of the kernel before this one
-  const int n_mtiles = a.tiles[0].x;
-  const ItemPlan plan = plan_items<TR::kGateUp>(a, n_mtiles);
+  const int n_mtiles = __shfl_sync(0xffffffffu, a.tiles[0].x, 0);
+  const ItemPlan plan = plan_items<TR::kGateUp>(a, n_mtiles, workers);
   const int n_whole = plan.n_whole;
   int n_mt_s = 0, n_shared = 0;
   if (kPair) {
-    n_mt_s = as.tiles[0].x;
+    n_mt_s = __shfl_sync(0xffffffffu, as.tiles[0].x, 0);
     n_shared = n_mt_s * as.n_ntiles * (TR::kGateUp ? 1 : as.k_splits);
   }
   const int n_items = plan.n_items + n_shared;
@@ -709,10 +754,10 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
     // ---------------------------------------------------------------- token-operand producer
     if (lane == 0) {
       RingPos p;
-      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+      for (int item = worker; item < n_items; item += workers) {
         const bool ok = is_shared(item)
-            ? load_operands<kS, S>(ts_a, ts_b0, ts_b1, as, shared_no(item), n_mt_s, n_shared, sA, sB, bars, p)
-            : load_operands<MODE, S>(tm_a, tm_b0, tm_b1, a, routed_no(item), n_mtiles, n_whole, sA, sB, bars, p);
+            ? load_operands<kS, S, CG>(ts_a, ts_b0, ts_b1, as, shared_no(item), n_mt_s, n_shared, sA, sB, bars, rank, p)
+            : load_operands<MODE, S, CG>(tm_a, tm_b0, tm_b1, a, routed_no(item), n_mtiles, n_whole, sA, sB, bars, rank, p);
         if (!ok) break;
       }
     }
@@ -720,22 +765,22 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
     // ---------------------------------------------------------------- packed-weight producer
     if (TR::kUnpack && lane == 0) {
       RingPos p;
-      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+      for (int item = worker; item < n_items; item += workers) {
         bool ok = true;
-        if (!is_shared(item)) ok = load_codes<MODE, kStagesP, kStageP>(tm_b0, tm_b1, a, routed_no(item), n_mtiles, n_whole, sP, bars, p);
-        else if (ModeTraits<kS>::kUnpack) ok = load_codes<kS, kStagesP, kStageP>(ts_b0, ts_b1, as, shared_no(item), n_mt_s, n_shared, sP, bars, p);
+        if (!is_shared(item)) ok = load_codes<MODE, kStagesP, kStageP, CG>(tm_b0, tm_b1, a, routed_no(item), n_mtiles, n_whole, sP, bars, rank, p);
+        else if (ModeTraits<kS>::kUnpack) ok = load_codes<kS, kStagesP, kStageP, CG>(ts_b0, ts_b1, as, shared_no(item), n_mt_s, n_shared, sP, bars, rank, p);
         if (!ok) break;
       }
     }
   } else if (warp == 2) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    if (rank == 0) {
       RingPos p;
       int local = 0;
-      for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++local) {
+      for (int item = worker; item < n_items; item += workers, ++local) {
         const bool ok = is_shared(item)
-            ? issue_mmas<kS, S, TR::kUnpack>(as, shared_no(item), n_shared, local, tmem_base, sA, sB, bars, p)
-            : issue_mmas<MODE, S, TR::kUnpack>(a, routed_no(item), n_whole, local, tmem_base, sA, sB, bars, p);
+            ? issue_mmas<kS, S, CG>(as, shared_no(item), n_shared, local, tmem_base, sA, sB, bars, p)
+            : issue_mmas<MODE, S, CG>(a, routed_no(item), n_whole, local, tmem_base, sA, sB, bars, p);
         if (!ok) break;
       }
     }
@@ -745,19 +790,19 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
       const int group = (warp - 4) >> 2;
       RingPos p, q;
       uint32_t step = 0;
-      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+      for (int item = worker; item < n_items; item += workers) {
         const bool ok = is_shared(item)
-            ? expand_codes<kS, S, kStagesP, kStageP>(as, shared_no(item), n_shared, group, genB, genP, bars, p, q, step)
-            : expand_codes<MODE, S, kStagesP, kStageP>(a, routed_no(item), n_whole, group, genB, genP, bars, p, q, step);
+            ? expand_codes<kS, S, kStagesP, kStageP, CG>(as, shared_no(item), n_shared, group, genB, genP, bars, p, q, step)
+            : expand_codes<MODE, S, kStagesP, kStageP, CG>(a, routed_no(item), n_whole, group, genB, genP, bars, p, q, step);
         if (!ok) break;
       }
     }
-  } else if (warp >= 12) {
+  } else if (warp >= kFirstEpilogueWarp) {
     // ---------------------------------------------------------------- epilogue
     int local = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++local) {
-      const bool ok = is_shared(item) ? write_out<kS>(as, shared_no(item), n_mt_s, n_shared, local, tmem_base, genE, bars)
-                                      : write_out<MODE>(a, routed_no(item), n_mtiles, n_whole, local, tmem_base, genE, bars);
+    for (int item = worker; item < n_items; item += workers, ++local) {
+      const bool ok = is_shared(item) ? write_out<kS, CG>(as, shared_no(item), n_mt_s, n_shared, local, tmem_base, genE, bars, rank)
+                                      : write_out<MODE, CG>(a, routed_no(item), n_mtiles, n_whole, local, tmem_base, genE, bars, rank);
       if (!ok) break;
     }
   }
@@ -766,26 +811,28 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
   drain_after_abort(abort_flag);
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync();             // neither CTA's shared memory and TMEM go while the other still works with them
   if (warp == 2) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc<CG>(tmem_base, kTmemCols);
   }
   if (threadIdx.x == 0) report_abort(abort_flag, a.status);
+  if (CG == 2) cluster_sync();
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int MODE, int CG>
+__global__ void __launch_bounds__(ModeTraits<MODE, CG>::kThreads, 1)
 umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
                  const __grid_constant__ CUtensorMap tm_b1, const UmmaArgs a) {
-  umma_cta<MODE, -1>(tm_a, tm_b0, tm_b1, a, tm_a, tm_b0, tm_b1, a);
+  umma_cta<MODE, -1, CG>(tm_a, tm_b0, tm_b1, a, tm_a, tm_b0, tm_b1, a);
 }
 template <int MODE, int SMODE>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(ModeTraits<MODE>::kThreads, 1)
 umma_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b0,
                  const __grid_constant__ CUtensorMap tm_b1, const UmmaArgs a, const __grid_constant__ CUtensorMap ts_a,
                  const __grid_constant__ CUtensorMap ts_b0, const __grid_constant__ CUtensorMap ts_b1, const UmmaArgs as) {
-  umma_cta<MODE, SMODE>(tm_a, tm_b0, tm_b1, a, ts_a, ts_b0, ts_b1, as);
+  umma_cta<MODE, SMODE, 1>(tm_a, tm_b0, tm_b1, a, ts_a, ts_b0, ts_b1, as);
 }
 
 // One CTA that runs the GEMM kernels' bounded wait to its limit: an mbarrier nothing ever arrives
@@ -855,19 +902,23 @@ static int pick_bn(int N) {
   return 128;
 }
 
-template <int MODE>
+template <int MODE, int CG = 1>
 static mote_status_t launch_umma(const CUtensorMap& ta, const CUtensorMap& tb0, const CUtensorMap& tb1,
                                  const UmmaArgs& a, int max_items, cudaStream_t stream, bool pdl) {
-  using TR = ModeTraits<MODE>;
-  static PerDeviceOnce attr_once;                  // one per MODE (this function is a template)
-  MOTE_CUDA_OK(set_max_dynamic_smem(attr_once, umma_gemm_kernel<MODE>, (int)TR::kSmem));
-  const int sms = device_sm_count();
-  const int grid = std::max(1, std::min(sms, max_items));
-  if (pdl) MOTE_CUDA_OK(launch_pdl(umma_gemm_kernel<MODE>, dim3(grid), dim3(kThreads), TR::kSmem, stream, ta, tb0, tb1, a));
-  else umma_gemm_kernel<MODE><<<grid, kThreads, TR::kSmem, stream>>>(ta, tb0, tb1, a);
+  using TR = ModeTraits<MODE, CG>;
+  static PerDeviceOnce attr_once;                  // one per MODE and CG (this function is a template)
+  MOTE_CUDA_OK(set_max_dynamic_smem(attr_once, umma_gemm_kernel<MODE, CG>, (int)TR::kSmem));
+  const int grid = CG * std::max(1, std::min(device_sm_count() / CG, max_items));
+  MOTE_CUDA_OK(launch_ex(umma_gemm_kernel<MODE, CG>, dim3(grid), dim3(TR::kThreads), TR::kSmem, stream, pdl, CG, ta, tb0, tb1, a));
   ++g_launch_count;
   MOTE_LAUNCH_OK();
   return MOTE_OK;
+}
+
+// Rows of the (first) weight map's box; load_weight_rows fetches one or two of them.
+static uint32_t weight_box_rows(int bn, bool gateup, int cg) {
+  if (cg == 1 || gateup) return std::min(bn, 128);
+  return bn == 256 ? 64 : bn / 2;
 }
 
 // Tensor maps and arguments of one GEMM.
@@ -876,21 +927,23 @@ struct GemmSetup {
   UmmaArgs a{};
 };
 
+// cg: CTAs per tile (row tiles of 128 * cg rows)
 static bool setup_ternary(GemmSetup& u, const TernaryGemmArgs& g, bool gateup, const int4* tiles, int max_mtiles,
-                          const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status) {
+                          const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status, int cg) {
   int bn = gateup ? 256 : pick_bn(g.N);
   // a down projection with few row tiles: the narrowest tiles (at least 64 wide) that are no more than the SMs (the
   // weights are the traffic here, and they are read once either way)
   if (!gateup) {
-    const int sms = device_sm_count();
+    const int workers = device_sm_count() / cg;
     for (int n = 64; n < bn; n += 32)
-      if (g.N % n == 0 && max_mtiles * (g.N / n) <= sms) bn = n;
+      if (g.N % n == 0 && max_mtiles * (g.N / n) <= workers) bn = n;
   }
-  // second weight map: the up matrix (gate/up), or the rows beyond 128 of a down tile
+  // second weight map: the up matrix (gate/up), or the rows beyond 128 of a down tile of one CTA
+  const uint32_t rows0 = weight_box_rows(bn, gateup, cg);
   if (!make_map_2d(&u.ta, g.qa, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.P, (uint64_t)g.K, 128, 128,
                    CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_map_2d(&u.tb0, g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N, (uint64_t)g.K / 4,
-                   std::min(bn, 128), 32, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+                   rows0, 32, CU_TENSOR_MAP_SWIZZLE_NONE) ||
       !make_map_2d(&u.tb1, gateup ? g.w1 : g.w0, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)g.E * g.N,
                    (uint64_t)g.K / 4, (gateup || bn <= 128) ? 128 : bn - 128, 32, CU_TENSOR_MAP_SWIZZLE_NONE))
     return false;
@@ -913,11 +966,14 @@ static bool setup_ternary(GemmSetup& u, const TernaryGemmArgs& g, bool gateup, c
 
 mote_status_t launch_ternary_umma(const TernaryGemmArgs& g, bool gateup, const int4* tiles, int max_mtiles,
                                   const int32_t* rowsum, uint32_t* beta_out_bits, uint32_t* status,
-                                  cudaStream_t stream, bool pdl) {
+                                  cudaStream_t stream, bool pdl, int cg) {
   if (g.P == 0) return MOTE_OK;
   GemmSetup u;
-  if (!setup_ternary(u, g, gateup, tiles, max_mtiles, rowsum, beta_out_bits, status)) return MOTE_ERR_CUDA;
+  if (!setup_ternary(u, g, gateup, tiles, max_mtiles, rowsum, beta_out_bits, status, cg)) return MOTE_ERR_CUDA;
   const int max_items = max_mtiles * u.a.n_ntiles;
+  if (cg == 2)
+    return gateup ? launch_umma<MODE_T_GATEUP, 2>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl)
+                  : launch_umma<MODE_T_DOWN, 2>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl);
   return gateup ? launch_umma<MODE_T_GATEUP>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl)
                 : launch_umma<MODE_T_DOWN>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl);
 }
@@ -935,17 +991,57 @@ int shared_down_k_splits(int64_t T, int N, int K) {
   return (int)std::max<int64_t>(splits, 1);
 }
 
+// ------------------------------------------------------------------------------------------------
+// One CTA per tile of 128 rows or a pair per tile of 256?  Per pipeline step a pair needs half the weight bytes, half of the
+// expansion and half of the weight operand's reads from shared memory in each SM, but its row tiles are twice as long, which
+// rounds an expert's rows up to 256, and half as many workers end in a longer last round.  So both are put as pipeline steps (a
+// step of the routed gate/up GEMM on single CTAs, 0.42 us, is the unit; the other rates are measured in that unit) times rounds.
+// us of the two GEMMs of the routed experts (gate/up + down), single CTAs / pairs: 2048 x 11008, 16 experts, top-2: 134 / 172 (768
+// tokens), 180 / 176 (960), 285 / 248 (2048); 4 experts, top-1: 96 / 80 (768); 896 x 4864, 4 experts: 54 / 60 (1024), 92 / 92 (2304),
+// 126 / 117 (4096); 512 x 2048, 16 experts: 62 / 68 (4096).  Of the shared ones: 2048 x 11008: 127 / 143 (1152: K splits fill one
+// round of single CTAs), 182 / 166 (1536); 256 x 512: 39 / 43 (8192).
+// ------------------------------------------------------------------------------------------------
+static double gemm_steps(double row_tiles, int n_tiles, double steps, int workers, bool halves, double per_step, double least) {
+  const double rounds = row_tiles * n_tiles / workers, whole = std::floor(rounds + 1e-9), tail = rounds - whole;
+  const double last = tail <= 1e-6 ? 0.0 : halves && tail <= 0.5 ? 0.6 : 1.0;
+  return (whole + last) * std::max(steps * per_step, least);      // least: a tile's epilogue, where K is short
+}
+int routed_ctas_per_tile(int64_t P, int E, int d, int f) {
+  double cost[2];
+  for (int cg = 1; cg <= 2; ++cg) {
+    const int workers = device_sm_count() / cg, bn = pick_bn(d);
+    const double row_tiles = double(P) / (128 * cg) + 0.5 * std::min<int64_t>(E, P);     // the router's choice is not known here
+    const double steps = gemm_steps(row_tiles, f / 128, d / 128, workers, false, cg == 1 ? 1.0 : 0.72, cg == 1 ? 14 : 12) +
+                         gemm_steps(row_tiles, d / bn, f / 128, workers, bn == 256, cg == 1 ? 0.9 : 0.75, 0);
+    cost[cg - 1] = steps + (cg == 1 ? 0 : 8);                       // clusters start later
+  }
+  return cost[1] < cost[0] ? 2 : 1;
+}
+int shared_ctas_per_tile(int64_t T, int d, int f, int k_splits) {
+  double cost[2];
+  for (int cg = 1; cg <= 2; ++cg) {
+    const int workers = device_sm_count() / cg, bn = pick_bn(d);
+    const double row_tiles = double((T + 128 * cg - 1) / (128 * cg));
+    const double steps = gemm_steps(row_tiles, f / 128, d / 64, workers, false, cg == 1 ? 0.93 : 0.85, 0) +
+                         gemm_steps(row_tiles, d / bn * k_splits, f / 64.0 / k_splits, workers, bn == 256 && k_splits == 1,
+                                    cg == 1 ? 1.1 : 1.03, 0);
+    cost[cg - 1] = steps + (cg == 1 ? 0 : 8);
+  }
+  return cost[1] < cost[0] ? 2 : 1;
+}
+
 static bool setup_shared(GemmSetup& u, const void* act, const SharedMat& w0, const SharedMat& w1, int bits, bool gateup,
                          int64_t T, int K, int N, void* out, const int4* tiles, uint32_t* status, const CombineArgs* comb,
-                         int k_splits) {
+                         int k_splits, int cg) {
   const int bn = gateup ? 256 : pick_bn(N);
+  const uint32_t rows0 = weight_box_rows(bn, gateup, cg);
   const uint32_t rows1 = (gateup || bn <= 128) ? 128 : bn - 128;
   if (!make_map_2d(&u.ta, act, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)T, (uint64_t)K, 128, 64,
                    CU_TENSOR_MAP_SWIZZLE_128B))
     return false;
   const void* wb1 = gateup ? w1.w : w0.w;
   if (bits == 16) {
-    if (!make_map_2d(&u.tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)N, (uint64_t)K, 128, 64,
+    if (!make_map_2d(&u.tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)N, (uint64_t)K, rows0, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map_2d(&u.tb1, wb1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (uint64_t)N, (uint64_t)K, rows1, 64,
                      CU_TENSOR_MAP_SWIZZLE_128B))
@@ -954,7 +1050,7 @@ static bool setup_shared(GemmSetup& u, const void* act, const SharedMat& w0, con
     // code rows as bytes: K (int8) or K/2 (4-bit) per row, 64 reduction elements per pipeline stage
     const uint64_t row_bytes = bits == 8 ? (uint64_t)K : (uint64_t)K / 2;
     const uint32_t box = bits == 8 ? 64 : 32;
-    if (!make_map_2d(&u.tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, row_bytes, 128, box,
+    if (!make_map_2d(&u.tb0, w0.w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, row_bytes, rows0, box,
                      CU_TENSOR_MAP_SWIZZLE_NONE) ||
         !make_map_2d(&u.tb1, wb1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, (uint64_t)N, row_bytes, rows1, box,
                      CU_TENSOR_MAP_SWIZZLE_NONE))
@@ -985,13 +1081,17 @@ static bool setup_shared(GemmSetup& u, const void* act, const SharedMat& w0, con
 mote_status_t launch_shared_umma(const void* act, const SharedMat& w0, const SharedMat& w1, int bits, bool gateup,
                                  int64_t T, int K, int N, void* out, const int4* tiles, int max_mtiles,
                                  uint32_t* status, const CombineArgs* comb, cudaStream_t stream, bool pdl,
-                                 int k_splits) {
+                                 int k_splits, int cg) {
   if (T == 0) return MOTE_OK;
   if (k_splits > 1 && (gateup || comb || !out)) return MOTE_ERR_SHAPE;
+  if (cg == 2 && bits != 16) return MOTE_ERR_SHAPE;
   GemmSetup u;
-  if (!setup_shared(u, act, w0, w1, bits, gateup, T, K, N, out, tiles, status, comb, k_splits)) return MOTE_ERR_CUDA;
+  if (!setup_shared(u, act, w0, w1, bits, gateup, T, K, N, out, tiles, status, comb, k_splits, cg)) return MOTE_ERR_CUDA;
   const UmmaArgs& a = u.a;
   const int max_items = max_mtiles * a.n_ntiles * a.k_splits;
+  if (cg == 2)
+    return gateup ? launch_umma<MODE_B_GATEUP, 2>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl)
+                  : launch_umma<MODE_B_DOWN, 2>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl);
   if (bits == 8)
     return gateup ? launch_umma<MODE_Q8_GATEUP>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl)
                   : launch_umma<MODE_Q8_DOWN>(u.ta, u.tb0, u.tb1, a, max_items, stream, pdl);
@@ -1004,7 +1104,8 @@ mote_status_t launch_shared_umma(const void* act, const SharedMat& w0, const Sha
 
 template <int MODE, int SMODE>
 static mote_status_t launch_pair(const GemmSetup& r, const GemmSetup& sh, int max_items, cudaStream_t stream, bool pdl) {
-  constexpr size_t smem = PairTraits<MODE, SMODE>::kSmem;
+  constexpr size_t smem = PairTraits<MODE, SMODE, 1>::kSmem;
+  constexpr int kThreads = PairTraits<MODE, SMODE, 1>::kThreads;
   static PerDeviceOnce attr_once;                  // one per pair
   MOTE_CUDA_OK(set_max_dynamic_smem(attr_once, umma_pair_kernel<MODE, SMODE>, (int)smem));
   const int grid = std::max(1, std::min(device_sm_count(), max_items));
@@ -1024,8 +1125,8 @@ mote_status_t launch_umma_pair(const TernaryGemmArgs& g, bool gateup, const int4
                                int max_mtiles_shared, uint32_t* status, cudaStream_t stream, bool pdl, int k_splits) {
   if (g.P == 0) return MOTE_OK;
   GemmSetup r, sh;
-  if (!setup_ternary(r, g, gateup, tiles_routed, max_mtiles_routed, rowsum, beta_out_bits, status) ||
-      !setup_shared(sh, act, w0, w1, bits, gateup, T, g.K, g.N, out, tiles_shared, status, nullptr, k_splits))
+  if (!setup_ternary(r, g, gateup, tiles_routed, max_mtiles_routed, rowsum, beta_out_bits, status, 1) ||
+      !setup_shared(sh, act, w0, w1, bits, gateup, T, g.K, g.N, out, tiles_shared, status, nullptr, k_splits, 1))
     return MOTE_ERR_CUDA;
   const int max_items = max_mtiles_routed * r.a.n_ntiles + max_mtiles_shared * sh.a.n_ntiles * sh.a.k_splits;
   if (bits == 8)

@@ -60,6 +60,14 @@ def test_c4_full_size_sampled(mote):
     assert rep["counts"].min() >= 0 and rep["counts"].sum() == 2 * 8192
 
 
+@pytest.mark.parametrize("d,f,E,k,T", [          # long enough for pairs of CTAs: down tiles of 256 (and halves), 224, 192 and 160 columns,
+    (1280, 4096, 5, 2, 2600), (896, 4864, 3, 2, 3071), (384, 9216, 2, 1, 4000), (640, 7168, 4, 1, 4500),
+    (1536, 4096, 7, 1, 2305), (384, 28672, 2, 1, 2047)])      # the shared expert alone; with K splits
+def test_pairs_of_ctas(mote, d, f, E, k, T):
+    rep = _sampled_parity(mote, synth.custom("pairs", d, f, E, k, T, 7000 + d + T), n_random=32, max_boundary_tokens=64)
+    assert rep["rel_fro"] < 5e-3
+
+
 @pytest.mark.parametrize("T", [1, 48, 333])
 def test_paper_configuration_top1_full_softmax_gate(mote, T):
     # the paper's 0.5B model layer: 1 shared + 4 routed experts, top-1, gate weight = P(x)_i of Eq. 3

@@ -96,7 +96,7 @@ def source_order():
     return order
 
 
-@pytest.mark.parametrize("stages,code_stages", [(3, 3), (3, 4)])     # INT8 codes; 2-bit and 4-bit ones
+@pytest.mark.parametrize("stages,code_stages", [(3, 3), (3, 4), (6, 6)])     # INT8 codes; 2-bit and 4-bit ones; pairs of CTAs
 def test_unpackers_meet_the_codes_of_their_own_step(stages, code_stages):
     for seed in range(400):
         walk(source_order(), stages, code_stages, 24, random.Random(seed))
