@@ -25,10 +25,10 @@
 // 0,4,8,12,1,5,...; the token operand is stored in the same order by the activation quantizer,
 // and an integer dot product does not depend on the order of its terms.
 //
-// Warp roles (640 threads): 0 TMA producer of the token operand (and of bf16 weights),
-// 1 TMA producer of packed weights, 2 MMA issuer + TMEM owner, 4-11 two groups of unpackers
-// that take alternate pipeline stages, 12-19 epilogue (two warps per TMEM lane quarter, each
-// owning half of the tile's columns).
+// Warp roles: 0 TMA producer of the token operand (and of bf16 weights), 1 TMA producer of packed weights, 2 MMA issuer and
+// TMEM owner, 4-11 two groups of unpackers that take alternate pipeline stages, 12 and up epilogue (eight or sixteen warps, an
+// equal number per TMEM lane quarter, which share the tile's columns).  Kernels with nothing to expand have their epilogue from
+// warp 4 on (see kEpiFirst, kEpiWarps).
 // Pairs of CTAs (CG = 2, clusters of two; long prefills, see routed_ctas_per_tile): a tile is 256 token rows, 128 in either
 // CTA, and cta_group::2 MMAs, issued by the first CTA, read half of the weight rows from each.  So either CTA fetches, expands and
 // keeps 128 weight rows instead of 256 for the same MMA work (32 KB per stage instead of 48, six stages instead of three), and an
@@ -53,7 +53,8 @@ namespace mote {
 using namespace ptx;
 
 enum { MODE_T_GATEUP = 0, MODE_T_DOWN = 1, MODE_B_GATEUP = 2, MODE_B_DOWN = 3,
-       MODE_Q8_GATEUP = 4, MODE_Q8_DOWN = 5, MODE_Q4_GATEUP = 6, MODE_Q4_DOWN = 7 };
+       MODE_Q8_GATEUP = 4, MODE_Q8_DOWN = 5, MODE_Q4_GATEUP = 6, MODE_Q4_DOWN = 7,
+       MODE_T_GATEUP_SHORT = 8 };
 
 constexpr int kBM = 128;
 constexpr int kStageA = kBM * 128;             // 16 KB: 128 rows x 128 B
@@ -61,8 +62,11 @@ constexpr int kStageB = 256 * 128;             // 32 KB: up to 256 rows x 128 B
 constexpr int kStagesTernary = 3, kStagesBf16 = 4, kStagesRtn = 3;
 constexpr int kStagesPaired = 6;               // half the weight rows per CTA: 32 KB per stage
 constexpr int kMaxStages = 6;
-constexpr int kFirstEpilogueWarp = 12;
 constexpr int kTmemCols = 512;
+// Up to this K a tile's epilogue (7 000 cycles on eight warps) takes longer than its MMAs (512 per 128 of K), so the ternary
+// gate/up GEMM on pairs of CTAs has sixteen epilogue warps there, at 72 registers (896 x 4864, 4096 tokens: 80 -> 75 us).  At
+// K = 2048 the MMAs hide eight warps' epilogue, and the extra warps take issue slots from the unpackers (435 -> 451 us).
+constexpr int kShortK = 1024;
 
 struct UmmaArgs {
   const int4* tiles;        // [0] = {n_mtiles,0,0,0}; [1+i] = {expert, row0, rows, 0}
@@ -99,8 +103,8 @@ struct __align__(8) PipeBarriers {
 // CG: CTAs per tile (see the head of this file)
 template <int MODE, int CG = 1>
 struct ModeTraits {
-  static constexpr bool kTernary = (MODE == MODE_T_GATEUP || MODE == MODE_T_DOWN);
-  static constexpr int kRtnBits = MODE >= MODE_Q4_GATEUP ? 4 : MODE >= MODE_Q8_GATEUP ? 8 : 0;
+  static constexpr bool kTernary = (MODE == MODE_T_GATEUP || MODE == MODE_T_DOWN || MODE == MODE_T_GATEUP_SHORT);
+  static constexpr int kRtnBits = kTernary ? 0 : MODE >= MODE_Q4_GATEUP ? 4 : MODE >= MODE_Q8_GATEUP ? 8 : 0;
   static constexpr bool kRtn = kRtnBits != 0;
   static constexpr bool kUnpack = kTernary || kRtn;       // weights reach shared memory as codes
   static constexpr bool kGateUp = (MODE % 2 == 0);
@@ -115,8 +119,11 @@ struct ModeTraits {
   // (bf16 gate/up only.  For the ternary gate/up, whose epilogue competes with the unpackers for
   // issue slots, staging -- with plain stores or with a TMA store -- measured slower than letting
   // every thread write its own 32 bytes.)
-  static constexpr int kEpiWarps = 8;
-  static constexpr int kThreads = (kFirstEpilogueWarp + kEpiWarps) * 32;
+  // bf16 weights need no unpackers, whose warps do the epilogue then.  The down projection, whose epilogue waits for the rows of
+  // y that it combines, has sixteen: all CTAs are in it at once after the last round (2048 x 11008, 2048 tokens: 86 -> 83 us).
+  static constexpr int kEpiFirst = kUnpack ? 12 : 4;
+  static constexpr int kEpiWarps = (MODE == MODE_B_DOWN || MODE == MODE_T_GATEUP_SHORT) ? 16 : 8;
+  static constexpr int kThreads = (kEpiFirst + kEpiWarps) * 32;
   static constexpr int kEpiCols = 32;
   static constexpr int kEpiPitch = kEpiCols * 2 + 16;
   static constexpr size_t kEpiStage = (kGateUp && !kTernary) ? size_t(8) * 32 * kEpiPitch : 0;
@@ -131,7 +138,7 @@ struct PairTraits {
   static constexpr int kStageB = mote::kStageB;
   using TR = ModeTraits<MODE>; using TS = ModeTraits<SMODE>;
   static constexpr bool kGateUp = TR::kGateUp, kUnpack = true;
-  static constexpr int kEpiWarps = TR::kEpiWarps, kThreads = TR::kThreads;
+  static constexpr int kEpiFirst = TR::kEpiFirst, kEpiWarps = TR::kEpiWarps, kThreads = TR::kThreads;
   static constexpr int kStages = kStagesTernary;
   static constexpr int kStageP = std::max(TR::kStageP, TS::kUnpack ? TS::kStageP : 0);
   static constexpr int kStagesP = TS::kRtnBits == 8 ? 3 : 4;
@@ -442,15 +449,16 @@ __device__ __forceinline__ bool expand_codes(const UmmaArgs& a, int item, int n_
   return true;
 }
 
-template <int MODE, int CG>
+// kFirst, kWarps: the epilogue warps of the CTA
+template <int MODE, int CG, int kFirst, int kWarps>
 __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mtiles, int n_whole, int local, uint32_t tmem_base,
                                           uint8_t* genE, PipeBarriers* bars, uint32_t rank) {
   using TR = ModeTraits<MODE, CG>;
   volatile int* abort_flag = &bars->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;                          // TMEM lane quarter this warp may read
-  constexpr int kParts = TR::kEpiWarps / 4;         // warps per lane quarter
-  const int part = (warp - kFirstEpilogueWarp) >> 2;   // which part of the tile's columns
+  constexpr int kParts = kWarps / 4;                // warps per lane quarter
+  const int part = (warp - kFirst) >> 2;            // which part of the tile's columns
   const int r_in_tile = q * 32 + lane;
   int4 tile; int n_tile, half;
   decode_item<TR::kGateUp>(a, item, n_mtiles, n_whole, tile, n_tile, half);
@@ -484,7 +492,7 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
     float hmax = 0.0f;                           // max |h| (before the bf16 rounding, which is monotonic)
     constexpr int kCols = TR::kEpiCols, kPitch = TR::kEpiPitch;
     constexpr int kLanesPerRow = kCols * 2 / 16, kRowsPerStore = 32 / kLanesPerRow;
-    uint8_t* stg = genE + (warp - kFirstEpilogueWarp) * 32 * kPitch;
+    uint8_t* stg = genE + (warp - kFirst) * 32 * kPitch;
 #pragma unroll 1
     for (int cr = part * (128 / kParts); cr < (part + 1) * (128 / kParts); cr += kCols) {
 #pragma unroll 1
@@ -583,7 +591,6 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
     const uint32_t acc_bias = 0x4B400000u - (uint32_t)rs;   // see glu_h2_fast_biased
     const int width = half < 0 ? a.bn : 128;
     const int col0 = n_tile * a.bn + (half > 0 ? 128 : 0);
-    const int cbeg = part * (width / kParts), cend = cbeg + width / kParts;
     const bool combine = !TR::kTernary && a.comb_out != nullptr;
     float cw[MOTE_MAX_TOPK];
     const float* cy[MOTE_MAX_TOPK];
@@ -596,7 +603,7 @@ __device__ __forceinline__ bool write_out(const UmmaArgs& a, int item, int n_mti
         }
     }
 #pragma unroll 1
-    for (int c = cbeg; c < cend; c += 16) {
+    for (int c = part * 16; c < width; c += kParts * 16) {
       uint32_t ra[16];
       tmem_ld_32x32b_x16(t_row + c, ra);
       tmem_wait_ld();
@@ -784,7 +791,7 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
         if (!ok) break;
       }
     }
-  } else if (warp >= 4 && warp < 12) {
+  } else if (TR::kUnpack && warp >= 4 && warp < 12) {
     // ---------------------------------------------------------------- code unpackers
     if (TR::kUnpack) {
       const int group = (warp - 4) >> 2;
@@ -797,12 +804,12 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
         if (!ok) break;
       }
     }
-  } else if (warp >= kFirstEpilogueWarp) {
+  } else if (warp >= TR::kEpiFirst) {
     // ---------------------------------------------------------------- epilogue
     int local = 0;
     for (int item = worker; item < n_items; item += workers, ++local) {
-      const bool ok = is_shared(item) ? write_out<kS, CG>(as, shared_no(item), n_mt_s, n_shared, local, tmem_base, genE, bars, rank)
-                                      : write_out<MODE, CG>(a, routed_no(item), n_mtiles, n_whole, local, tmem_base, genE, bars, rank);
+      const bool ok = is_shared(item) ? write_out<kS, CG, TR::kEpiFirst, TR::kEpiWarps>(as, shared_no(item), n_mt_s, n_shared, local, tmem_base, genE, bars, rank)
+                                      : write_out<MODE, CG, TR::kEpiFirst, TR::kEpiWarps>(a, routed_no(item), n_mtiles, n_whole, local, tmem_base, genE, bars, rank);
       if (!ok) break;
     }
   }
@@ -972,7 +979,8 @@ mote_status_t launch_ternary_umma(const TernaryGemmArgs& g, bool gateup, const i
   if (!setup_ternary(u, g, gateup, tiles, max_mtiles, rowsum, beta_out_bits, status, cg)) return MOTE_ERR_CUDA;
   const int max_items = max_mtiles * u.a.n_ntiles;
   if (cg == 2)
-    return gateup ? launch_umma<MODE_T_GATEUP, 2>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl)
+    return gateup && g.K <= kShortK ? launch_umma<MODE_T_GATEUP_SHORT, 2>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl)
+           : gateup ? launch_umma<MODE_T_GATEUP, 2>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl)
                   : launch_umma<MODE_T_DOWN, 2>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl);
   return gateup ? launch_umma<MODE_T_GATEUP>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl)
                 : launch_umma<MODE_T_DOWN>(u.ta, u.tb0, u.tb1, u.a, max_items, stream, pdl);
