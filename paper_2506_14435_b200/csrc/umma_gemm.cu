@@ -288,6 +288,19 @@ __device__ __forceinline__ bool load_operands(const CUtensorMap& tm_a, const CUt
   return true;
 }
 
+// After its last item the token producer walks the ring once more: the commits of the last S steps have arrived at this CTA's
+// `empty` barriers before it may leave.  Nobody else waits for them (the epilogue waits for another commit, and arrivals of two
+// commits have no order), and in a pair they come from the other CTA, whose closing cluster barrier orders its threads'
+// accesses but not asynchronous arrivals.
+template <int S>
+__device__ __forceinline__ bool await_last_commits(PipeBarriers* bars, RingPos p) {
+  for (int i = 0; i < S; ++i) {
+    if (!mbar_wait(smem_u32(&bars->empty[p.stage]), p.phase ^ 1, &bars->abort_flag)) return false;
+    p.next(S);
+  }
+  return true;
+}
+
 // weight codes (a pair: either CTA the codes of its half of the weight rows, on its own barrier)
 template <int MODE, int kStagesP, int kStageP, int CG>
 __device__ __forceinline__ bool load_codes(const CUtensorMap& tm_b0, const CUtensorMap& tm_b1, const UmmaArgs& a, int item, int n_mtiles, int n_whole,
@@ -761,12 +774,12 @@ __device__ __forceinline__ void umma_cta(const CUtensorMap& tm_a, const CUtensor
     // ---------------------------------------------------------------- token-operand producer
     if (lane == 0) {
       RingPos p;
-      for (int item = worker; item < n_items; item += workers) {
-        const bool ok = is_shared(item)
+      bool ok = true;
+      for (int item = worker; ok && item < n_items; item += workers)
+        ok = is_shared(item)
             ? load_operands<kS, S, CG>(ts_a, ts_b0, ts_b1, as, shared_no(item), n_mt_s, n_shared, sA, sB, bars, rank, p)
             : load_operands<MODE, S, CG>(tm_a, tm_b0, tm_b1, a, routed_no(item), n_mtiles, n_whole, sA, sB, bars, rank, p);
-        if (!ok) break;
-      }
+      if (ok) (void)await_last_commits<S>(bars, p);
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- packed-weight producer
