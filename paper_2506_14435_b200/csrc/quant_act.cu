@@ -44,7 +44,7 @@ __device__ __forceinline__ void scan_block_counts(const QuantActArgs& a, InlineS
   __syncthreads();
   if (warp == 0) {
     const int c0 = lane < E ? sc.count[lane] : 0, c1 = lane + 32 < E ? sc.count[lane + 32] : 0;
-    const int tr = 128 * a.cg_routed, n0 = (c0 + tr - 1) / tr, n1 = (c1 + tr - 1) / tr;
+    const int tr = 128 * a.cg_routed, lg = 6 + a.cg_routed, n0 = (c0 + tr - 1) >> lg, n1 = (c1 + tr - 1) >> lg;
     const int r0 = scan_inclusive(c0, lane), t0 = scan_inclusive(n0, lane);
     const int r1 = scan_inclusive(c1, lane) + __shfl_sync(0xffffffffu, r0, 31);
     const int t1 = scan_inclusive(n1, lane) + __shfl_sync(0xffffffffu, t0, 31);
@@ -58,7 +58,7 @@ __device__ __forceinline__ void scan_block_counts(const QuantActArgs& a, InlineS
         a.offsets_out[E] = r1;
         a.tiles_routed[0] = make_int4(t1, 0, 0, 0);
       }
-      const int T = (int)a.T, ts = 128 * a.cg_shared, n = (T + ts - 1) / ts;
+      const int T = (int)a.T, ts = 128 * a.cg_shared, n = (T + ts - 1) >> (6 + a.cg_shared);
       for (int i = lane; i < n; i += 32) a.tiles_shared[1 + i] = make_int4(0, i * ts, min(ts, T - i * ts), 0);
       if (lane == 0) a.tiles_shared[0] = make_int4(n, 0, 0, 0);
     }
