@@ -354,6 +354,11 @@ mote_status_t mote_int8_mma_peak(void* ws, int n_batches, double* ops_host, void
 /* Number of kernels the last mote_moe_forward call on this thread enqueued. */
 int mote_last_launch_count(void);
 
+/* Diagnostic: the output tile of one GEMM of the last mote_moe_forward call on this thread, as rows << 16 | columns; 0 if that
+ * GEMM was not a tensor-core launch of its own.  gemm: 0 routed gate/up, 1 routed down, 2 shared gate/up, 3 shared down.  Tiles of
+ * 128 rows are the work of one thread block, tiles of 256 rows that of a pair. */
+int mote_last_gemm_tile(int gemm);
+
 #ifdef __cplusplus
 }
 #endif

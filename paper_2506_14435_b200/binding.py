@@ -90,6 +90,8 @@ lib.mote_int8_mma_peak.restype = C.c_int
 lib.mote_int8_mma_peak.argtypes = [C.c_void_p, C.c_int, C.POINTER(C.c_double), C.c_void_p]
 lib.mote_last_launch_count.restype = C.c_int
 lib.mote_last_launch_count.argtypes = []
+lib.mote_last_gemm_tile.restype = C.c_int
+lib.mote_last_gemm_tile.argtypes = [C.c_int]
 
 
 class MoteError(RuntimeError):

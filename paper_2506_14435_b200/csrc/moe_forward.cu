@@ -11,6 +11,7 @@
 namespace mote {
 
 thread_local int g_launch_count = 0;
+thread_local int g_gemm_tile[4] = {};
 
 // Set while mote_stack_forward runs its layers: the stack clears the device status word once, at
 // its start, and the layer calls inside it leave the word alone, so that a bounded wait that ran
@@ -205,6 +206,8 @@ extern "C" size_t mote_host_staging_bytes(int d, int64_t T_max) {
 
 extern "C" int mote_last_launch_count(void) { return g_launch_count; }
 
+extern "C" int mote_last_gemm_tile(int gemm) { return gemm >= 0 && gemm < 4 ? g_gemm_tile[gemm] : 0; }
+
 extern "C" mote_status_t mote_device_status(void* ws, void* stream_) {
   if (!ws) return MOTE_ERR_NULL;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
@@ -229,6 +232,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
                                           void* out, const mote_taps_t* taps, void* ws, size_t ws_bytes,
                                           void* stream_) {
   g_launch_count = 0;
+  for (int& tile : g_gemm_tile) tile = 0;
   if (!L) return MOTE_ERR_NULL;
   const int d = L->d, f = L->f, E = L->E, k = L->k;
   if (!shape_ok(d, f, E, k) || T < 0 || T > (int64_t(1) << 24)) return MOTE_ERR_SHAPE;

@@ -120,6 +120,8 @@ mote_status_t launch_umma_pair(const TernaryGemmArgs& g, bool gateup, const int4
 // Diagnostic: one CTA waits on an mbarrier that nothing arrives at, with the GEMM kernels' bounded
 // wait and teardown; after limit_ns it raises *status and returns.
 mote_status_t launch_bounded_wait_selftest(uint32_t* status, uint64_t limit_ns, cudaStream_t stream);
+// Tiles of the tensor-core GEMMs of the thread's last forward call that were launches of their own (see mote_last_gemm_tile).
+extern thread_local int g_gemm_tile[4];
 constexpr int64_t kMaxPartialRows = 4096;
 int shared_down_k_splits(int64_t T, int N, int K);
 // CTAs per tile (1 or 2) of the routed experts' and of the shared expert's two GEMMs where each is a launch of its own.

@@ -942,6 +942,7 @@ static mote_status_t launch_umma(const CUtensorMap& ta, const CUtensorMap& tb0, 
   const int grid = CG * std::max(1, std::min(device_sm_count() / CG, max_items));
   MOTE_CUDA_OK(launch_ex(umma_gemm_kernel<MODE, CG>, dim3(grid), dim3(TR::kThreads), TR::kSmem, stream, pdl, CG, ta, tb0, tb1, a));
   ++g_launch_count;
+  g_gemm_tile[(TR::kTernary ? 0 : 2) + (TR::kGateUp ? 0 : 1)] = (kBM * CG) << 16 | a.bn;
   MOTE_LAUNCH_OK();
   return MOTE_OK;
 }

@@ -21,7 +21,7 @@ def mote():
     return m
 
 
-def _sampled_parity(mote, wl, n_random, max_boundary_tokens, shared_bits=16):
+def _sampled_parity(mote, wl, n_random, max_boundary_tokens, shared_bits=16, residual_bits=None):
     master = synth.master_layer(wl)
     layer_or = O.build_layer(master)
     layer_gpu = mote.MoteLayer.from_master(master)
@@ -38,7 +38,7 @@ def _sampled_parity(mote, wl, n_random, max_boundary_tokens, shared_bits=16):
         rng = np.random.default_rng(wl.seed)
         toks = np.sort(rng.choice(toks, size=max_boundary_tokens + n_random, replace=False))
     toks = toks[~r["near_tie"][toks]]          # a near tie may legitimately move a token to another expert
-    rep = check_forward(mote, layer_gpu, layer_or, x_bits, token_subset=toks)
+    rep = check_forward(mote, layer_gpu, layer_or, x_bits, residual_bits=residual_bits, token_subset=toks)
     assert rep["tokens"] >= min(64, wl.T)
     return rep
 
@@ -60,12 +60,34 @@ def test_c4_full_size_sampled(mote):
     assert rep["counts"].min() >= 0 and rep["counts"].sum() == 2 * 8192
 
 
-@pytest.mark.parametrize("d,f,E,k,T", [          # long enough for pairs of CTAs: down tiles of 256 (and halves), 224, 192 and 160 columns,
-    (1280, 4096, 5, 2, 2600), (896, 4864, 3, 2, 3071), (384, 9216, 2, 1, 4000), (640, 7168, 4, 1, 4500),
-    (1536, 4096, 7, 1, 2305), (384, 28672, 2, 1, 2047)])      # the shared expert alone; with K splits
-def test_pairs_of_ctas(mote, d, f, E, k, T):
-    rep = _sampled_parity(mote, synth.custom("pairs", d, f, E, k, T, 7000 + d + T), n_random=32, max_boundary_tokens=64)
+# Calls that run on pairs of CTAs.  tiles: rows x columns of the routed and of the shared down projection's tiles (256 rows: a pair);
+# halves: tiles of the last round that are cut in two, routed and shared, on the 148 SMs of a B200 (see plan_items)
+@pytest.mark.parametrize("d,f,E,k,T,bits,tiles,halves", [
+    (1280, 4096, 5, 2, 2600, 16, ((256, 256), (256, 256)), (0, 0)),
+    (1280, 3072, 2, 1, 3900, 16, ((256, 256), (256, 256)), (6, 6)),
+    (768, 4096, 3, 2, 3333, 4, ((256, 256), (128, 256)), (7, 0)),      # sixteen epilogue warps; codes expanded ahead of single CTAs
+    (896, 4864, 3, 2, 3071, 16, ((256, 224), (256, 224)), (0, 0)),
+    (384, 8192, 2, 2, 3500, 16, ((256, 192), (256, 192)), (0, 0)),
+    (640, 7168, 4, 1, 4500, 16, ((256, 160), (256, 160)), (0, 0)),
+    (1408, 4096, 3, 2, 1800, 8, ((256, 128), (256, 128)), (0, 0)),      # codes expanded ahead of pairs
+    (384, 9216, 2, 1, 4000, 16, ((256, 96), (256, 192)), (0, 0)),
+    (384, 28672, 2, 1, 2047, 16, ((256, 64), (256, 192)), (0, 0)),      # the shared one with K splits
+    (1536, 4096, 7, 1, 2305, 16, ((128, 256), (256, 256)), (0, 0)),     # the shared expert alone
+    (3200, 512, 2, 2, 500, 16, ((256, 160), (128, 160)), (0, 0)),       # tables written by the CTAs of Q_a(x): the routed experts alone
+    (2432, 4608, 2, 1, 500, 16, ((256, 128), (256, 128)), (0, 0))])     # both
+def test_pairs_of_ctas(mote, d, f, E, k, T, bits, tiles, halves):
+    wl = synth.custom("pairs", d, f, E, k, T, 7000 + d + T)
+    residual = O.f32_to_bf16_rn(np.random.default_rng(d + T).standard_normal((T, d)).astype(np.float32)) if T % 2 else None
+    rep = _sampled_parity(mote, wl, n_random=64, max_boundary_tokens=64, shared_bits=bits, residual_bits=residual)
     assert rep["rel_fro"] < 5e-3
+    ran = [divmod(mote.lib.mote_last_gemm_tile(i), 1 << 16) for i in range(4)]
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert (ran[1], ran[3]) == tiles and [ran[0][0], ran[2][0]] == [ran[1][0], ran[3][0]]
+        for rows, (tile_rows, width), cut in ((rep["counts"], tiles[0], halves[0]), ([T], tiles[1], halves[1])):
+            workers = 148 * 128 // tile_rows
+            tail = sum(-(-int(n) // tile_rows) for n in rows) * (d // width) % workers
+            assert cut == (tail if width == 256 and 2 * tail <= workers else 0)
+    assert 256 in (ran[1][0], ran[3][0])
 
 
 @pytest.mark.parametrize("T", [1, 48, 333])
