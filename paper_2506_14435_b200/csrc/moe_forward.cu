@@ -369,33 +369,31 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   mote_status_t st;
   // device status word: cleared by the router kernel where the tensor-core router runs (one
   // operation less on the stream), else by a memset
-  const bool router_clears = !g_keep_status && tensor && (d % 32 == 0);
+  const bool router_clears = !g_keep_status && tensor;
   if (!g_keep_status && !router_clears) MOTE_CUDA_OK(cudaMemsetAsync(status, 0, 4, stream));
   stage_mark(0, stream);
   // S1 router, S2 dispatch
-  // block-wise dispatch: the tensor-core router (d % 32 == 0) leaves per-block expert counts, a small
+  // tensor path, block-wise dispatch: the tensor-core router leaves per-block expert counts, a small
   // scan turns them into bases, and Q_a(x) derives every pair's sorted row itself
-  const bool blockwise = tensor && (d % 32 == 0);
   auto* blk_hist = reinterpret_cast<int32_t*>(base + pl.blk_hist);
   auto* blk_base = reinterpret_cast<int32_t*>(base + pl.blk_base);
   const int n_blk = (int)((T + kRouteBlockTokens - 1) / kRouteBlockTokens);
   st = launch_route_topk(x, T, d, L->Wr, L->router_bias, E, k, L->norm_topk, topk_idx, topk_w, nullptr,
-                         blockwise ? blk_hist : nullptr, stream, router_clears ? status : nullptr);
+                         tensor ? blk_hist : nullptr, stream, router_clears ? status : nullptr);
   if (st) return st;
   stage_mark(1, stream);
-  const bool inline_scan = blockwise && n_blk <= kInlineScanBlocks;   // few blocks: done by the CTAs of Q_a(x)
+  const bool inline_scan = tensor && n_blk <= kInlineScanBlocks;   // few blocks: done by the CTAs of Q_a(x)
   st = inline_scan ? MOTE_OK
-       : blockwise ? launch_dispatch_scan(blk_hist, n_blk, E, offsets, blk_base, tiles_routed, cg_routed, tiles_shared, cg_shared, T,
+       : tensor    ? launch_dispatch_scan(blk_hist, n_blk, E, offsets, blk_base, tiles_routed, cg_routed, tiles_shared, cg_shared, T,
                                           stream)
-                   : launch_dispatch(topk_idx, P, E, offsets, perm, inv, tensor ? tiles_routed : nullptr,
-                                   tensor ? tiles_shared : nullptr, T, stream);
+                   : launch_dispatch(topk_idx, P, E, offsets, perm, inv, stream);
   if (st) return st;
   stage_mark(2, stream);
   // S3 Q_a(x), written once per selected expert into the expert-sorted rows
   QuantActArgs qa{};
   qa.x = x; qa.T = T; qa.d = d; qa.ldx = d; qa.q = qx; qa.beta = beta_x; qa.rowsum = rowsum_x;
   qa.perm = perm; qa.k = k; qa.interleave = interleave;
-  if (blockwise) {
+  if (tensor) {
     if (inline_scan) {
       qa.blk_hist = blk_hist; qa.offsets_out = offsets; qa.tiles_routed = tiles_routed; qa.tiles_shared = tiles_shared;
       qa.cg_routed = cg_routed; qa.cg_shared = cg_shared;
@@ -405,7 +403,7 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
     qa.topk_idx = topk_idx; qa.E = E; qa.n_blk = n_blk; qa.perm_out = perm; qa.inv_out = inv;
     qa.zero_u32 = reinterpret_cast<uint32_t*>(beta_h); qa.zero_i32 = rowsum_h;
   }
-  const bool pdl = blockwise;    // from here on every kernel is a programmatic dependent of the one before
+  const bool pdl = tensor;    // from here on every kernel is a programmatic dependent of the one before
   st = launch_quant_act(qa, true, stream);
   if (st) return st;
   stage_mark(3, stream);
@@ -431,8 +429,6 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
   g1.qa = qx; g1.beta = beta_x; g1.offsets = offsets; g1.w0 = L->gate_packed; g1.w1 = L->up_packed;
   g1.alpha0 = L->alpha_gate; g1.alpha1 = L->alpha_up; g1.E = E; g1.N = f; g1.K = d; g1.P = P;
   g1.h_bf16 = h; g1.acc0_tap = taps ? taps->acc_gate : nullptr; g1.acc1_tap = taps ? taps->acc_up : nullptr;
-  if (tensor && !blockwise)   // beta_h (atomicMax target) and rowsum_h (atomicAdd target) are adjacent
-    MOTE_CUDA_OK(cudaMemsetAsync(beta_h, 0, (pl.rowsum_h - pl.beta_h) + size_t(P) * 4, stream));
   st = pair     ? launch_umma_pair(g1, true, tiles_routed, max_mtiles_routed, rowsum_x, reinterpret_cast<uint32_t*>(beta_h), x,
                                    xg, xu, x_bits, T, hs, tiles_shared, max_mtiles_shared, status, stream, pdl, 1)
        : tensor ? launch_ternary_umma(g1, true, tiles_routed, max_mtiles_routed, rowsum_x,

@@ -144,7 +144,6 @@ extern thread_local int g_launch_count;
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ float bf16_lo(uint32_t packed2) { return __uint_as_float(packed2 << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t packed2) { return __uint_as_float(packed2 & 0xFFFF0000u); }
-__device__ __forceinline__ float bf16_bits_to_f32(uint16_t b) { return __uint_as_float(uint32_t(b) << 16); }
 
 // round-to-nearest-even fp32 -> bf16 bits (finite inputs)
 __device__ __forceinline__ uint32_t f32_to_bf16_bits(float x) {

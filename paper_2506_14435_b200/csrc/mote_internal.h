@@ -47,15 +47,12 @@ mote_status_t launch_route_topk(const void* x, int64_t T, int d, const float* Wr
 // zero_word (optional, tensor-core kernel only): a word the kernel's first thread sets to zero.
 
 // Stable grouping of the T*k pairs by expert: offsets[E+1], perm[P] (pair -> row), inv[P] (row -> pair).
-// Optionally also writes the 128-row tile tables of the tensor-core GEMMs ([0] = {count},
-// [1+i] = {expert, first row, rows}); tiles_routed needs 1 + P/128 + E entries, tiles_shared
-// 1 + ceil(T/128).
 mote_status_t launch_dispatch(const int32_t* idx, int64_t P, int E, int32_t* offsets, int32_t* perm,
-                              int32_t* inv, int4* tiles_routed, int4* tiles_shared, int64_t T,
-                              cudaStream_t stream);
+                              int32_t* inv, cudaStream_t stream);
 
-// Block-wise variant: offsets, per-block bases and the tile tables (of 128 * cg rows per tile) from the router's block
-// histograms.
+// Block-wise variant for the tensor path: offsets, per-block bases and the GEMMs' tile tables (of 128 * cg rows per tile) from
+// the router's block histograms.  A table: [0] = {count}, [1+i] = {expert, first row, rows}; tiles_routed needs 1 + P/128 + E
+// entries, tiles_shared 1 + ceil(T/128).
 mote_status_t launch_dispatch_scan(const int32_t* blk_hist, int n_blk, int E, int32_t* offsets, int32_t* blk_base,
                                    int4* tiles_routed, int cg_routed, int4* tiles_shared, int cg_shared, int64_t T,
                                    cudaStream_t stream);

@@ -124,23 +124,9 @@ __device__ __forceinline__ void ld_global_v8(const void* p, uint32_t (&v)[8]) {
                : "memory");
 }
 
-// 2-D tiled store shared -> global (bulk async-group completion).  x must be a multiple of 16
-// bytes worth of elements; neither coordinate may be negative.
-__device__ __forceinline__ void tma_store_2d(const void* tmap, uint32_t smem_src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                   reinterpret_cast<uint64_t>(tmap)),
-               "r"(x), "r"(y), "r"(smem_src)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// all committed bulk groups of this thread have finished READING their shared-memory source
-__device__ __forceinline__ void bulk_wait_group_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// ... and have completed entirely
-__device__ __forceinline__ void bulk_wait_group0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // ------------------------------------------------------------------ tcgen05 / TMEM
-// CG: CTAs that work on one tile (cta_group::1 or ::2); one value for all tcgen05 instructions of a kernel.  With two, alloc
-// and dealloc are issued by one warp of either CTA.
+// CG: CTAs that work on one tile (cta_group::1 or ::2); one value for all tcgen05 instructions of a kernel.  With two, one warp
+// of each CTA issues alloc and dealloc.
 template <int CG = 1>
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_result, uint32_t ncols) {
   if (CG == 1)
@@ -208,21 +194,8 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
                  : "memory");
 }
 
-// 32 lanes x 32 consecutive 32-bit columns -> 32 registers per thread (lane i of the warp reads
+// 32 lanes x 16 consecutive 32-bit columns -> 16 registers per thread (lane i of the warp reads
 // TMEM lane base+i).
-__device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-
 __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "

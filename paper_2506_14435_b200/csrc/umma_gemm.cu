@@ -1142,11 +1142,8 @@ static mote_status_t launch_pair(const GemmSetup& r, const GemmSetup& sh, int ma
   static PerDeviceOnce attr_once;                  // one per pair
   MOTE_CUDA_OK(set_max_dynamic_smem(attr_once, umma_pair_kernel<MODE, SMODE>, (int)smem));
   const int grid = std::max(1, std::min(device_sm_count(), max_items));
-  if (pdl)
-    MOTE_CUDA_OK(launch_pdl(umma_pair_kernel<MODE, SMODE>, dim3(grid), dim3(kThreads), smem, stream, r.ta, r.tb0, r.tb1, r.a,
-                            sh.ta, sh.tb0, sh.tb1, sh.a));
-  else
-    umma_pair_kernel<MODE, SMODE><<<grid, kThreads, smem, stream>>>(r.ta, r.tb0, r.tb1, r.a, sh.ta, sh.tb0, sh.tb1, sh.a);
+  MOTE_CUDA_OK(launch_ex(umma_pair_kernel<MODE, SMODE>, dim3(grid), dim3(kThreads), smem, stream, pdl, 1, r.ta, r.tb0, r.tb1, r.a,
+                         sh.ta, sh.tb0, sh.tb1, sh.a));
   ++g_launch_count;
   MOTE_LAUNCH_OK();
   return MOTE_OK;
