@@ -50,6 +50,10 @@ struct Plan {
 // layer to bf16 in the workspace (one streaming pass) and runs the plain bf16 GEMMs on them; below,
 // the GEMM expands the codes tile by tile in shared memory (less weight traffic, more work per row tile).
 constexpr int64_t kExpandMinTokens = 768;
+// The weight stream up to this many tokens.  us per layer, stream / GEMMs (bf16 shared expert; 4 experts top-1, 16 experts top-2): 2048 x
+// 11008 at 24 tokens 85 / 118, 159 / 229, at 32 91 / 111, 163 / 164, at 40 155 / 109, 278 / 165; 1536 x 8960 at 32 68 / 87, 115 / 149, at
+// 40 107 / 88, 189 / 143; 896 x 4864 at 32 40 / 53, 64 / 75, at 40 54 / 53, 95 / 74 (above 32 tokens the stream needs eight column tiles,
+// with half as many warps per SM).  INT8 and INT4 likewise, but for 2048 x 11008, INT4, 8 or 16 experts at 32 tokens (127 / 122, 172 / 162).
 constexpr int64_t kStreamAutoMaxTokens = 32;
 // Short prefills with bf16 operands for the shared expert run the routed and the shared GEMM of a step as one launch up to
 // this many multiply-adds of the shared gate projection (T * d * f): 975 tokens at 2048 x 11008.
@@ -350,12 +354,13 @@ extern "C" mote_status_t mote_moe_forward(const mote_layer_t* L, const void* x, 
 
   const bool expands = sh_rtn && tensor && T >= kExpandMinTokens && ws_bytes >= pl.total_expanded;   // see expand_shared
   // Few row tiles (the shared down projection is cut along K): the routed and the shared GEMM of a step both end in a
-  // partly filled round of tiles, so they are one launch, which also saves two.  Layers apart / as pairs: 256 x 512, 64
-  // tokens, 43.0 us in nine launches / 27.5 in six; 1536 x 8960, 8 experts, top-2: 116 / 99 (64 tokens), 152 / 147 (512),
-  // 200 / 194 (896), 261 / 257 (1408); 896 x 4864: 134 / 126 (1408).  A bf16 tile has three pipeline stages in a pair and
-  // four by itself, which shows once the shared GEMMs are long, hence kPairMaxWork: 2048 x 11008, 4 experts, top-1: 184 /
-  // 185 (640), 223 / 215 (896), 247 / 254 (1024), 268 / 279 (1152).  Tiles of RTN codes have three either way: 4096 x 14336,
-  // INT8, 384 tokens: 384 / 365.  With more row tiles yet, the shared down projection's epilogue does the combine, for
+  // partly filled round of tiles, so they are one launch, which also saves two.  us per layer, GEMMs apart (on pairs of CTAs
+  // where those are chosen) / as one launch: 256 x 512, 64 tokens, 39 in nine launches / 29 in six; 1536 x 8960, 8 experts, top-2: 109 /
+  // 101 (64 tokens), 151 / 145 (512), 197 / 197 (896), 260 / 253 (1408); 896 x 4864, 4 experts: 92 / 81 (512), 134 / 130 (1408).  A bf16
+  // tile has three pipeline stages in a pair and four or six by itself, which shows once the shared GEMMs are long, hence
+  // kPairMaxWork: 2048 x 11008, 4 experts, top-1: 151 / 148 (384), 181 / 187 (640), 219 / 215 (896), 210 / 230 (1024), 257 / 272 (1152);
+  // 16 experts, top-2: 248 / 249 (640), 321 / 334 (960).  Tiles of RTN codes have three either way: 4096 x 14336, INT8, 384 tokens:
+  // 355 / 344.  With more row tiles yet, the shared down projection's epilogue does the combine, for
   // which the routed one has to be complete.
   const int k_splits = tensor ? shared_down_k_splits(T, d, f) : 1;
   const bool codes = sh_rtn && !expands;

@@ -33,8 +33,8 @@
 // CTA, and cta_group::2 MMAs, issued by the first CTA, read half of the weight rows from each.  So either CTA fetches, expands and
 // keeps 128 weight rows instead of 256 for the same MMA work (32 KB per stage instead of 48, six stages instead of three), and an
 // SM's shared memory moves 72 KB per step instead of 112 in the 512 cycles that the step's MMAs take.  The second CTA's copies and
-// announcements go to the first one's `full` barriers; commits arrive at both.  2048 x 11008, 8192 tokens, 16 experts: routed
-// gate/up 595 -> 435 us (3 400 TOP/s), routed down 300 -> 224.  Half of that is the issue loop (see issue_mmas).
+// announcements go to the first one's `full` barriers; commits arrive at both.  2048 x 11008, 8192 tokens, 16 experts, both builds in
+// turn: routed gate/up 643 -> 477 us (3 100 TOP/s), routed down 315 -> 241.  Half of that is the issue loop (see issue_mmas).
 //
 // Two accumulator buffers of 256 TMEM columns let the epilogue of one tile overlap the MMAs of
 // the next.  Every mbarrier wait is bounded; on expiry the CTA raises a status word and leaves.
@@ -63,9 +63,11 @@ constexpr int kStagesTernary = 3, kStagesBf16 = 4, kStagesRtn = 3;
 constexpr int kStagesPaired = 6;               // half the weight rows per CTA: 32 KB per stage
 constexpr int kMaxStages = 6;
 constexpr int kTmemCols = 512;
-// Up to this K a tile's epilogue (7 000 cycles on eight warps) takes longer than its MMAs (512 per 128 of K), so the ternary
-// gate/up GEMM on pairs of CTAs has sixteen epilogue warps there, at 72 registers (896 x 4864, 4096 tokens: 80 -> 75 us).  At
-// K = 2048 the MMAs hide eight warps' epilogue, and the extra warps take issue slots from the unpackers (435 -> 451 us).
+// Up to this K a tile's epilogue (7 000 cycles on eight warps) takes clearly longer than its MMAs (512 per 128 of K), so the ternary
+// gate/up GEMM on pairs of CTAs has sixteen epilogue warps there, at 72 registers.  Where the MMAs hide eight warps' epilogue, the
+// extra warps only take issue slots from the unpackers.  f = 4096, 4 experts, top-2, 4096 tokens, eight / sixteen warps: 74 / 68 us at
+// K = 1024, 74 / 69 (1152), 77 / 72 (1280), 79 / 75 (1408), 80 / 78.5 (1536), 85 / 87 (1792), 92 / 95 (2048); 896 x 4864 80 / 74.5.
+// The line was drawn between K = 896 and 2048; by these figures it could lie at 1536.
 constexpr int kShortK = 1024;
 
 struct UmmaArgs {
@@ -1029,10 +1031,15 @@ int shared_down_k_splits(int64_t T, int N, int K) {
 // expansion and half of the weight operand's reads from shared memory in each SM, but its row tiles are twice as long, which
 // rounds an expert's rows up to 256, and half as many workers end in a longer last round.  So both are put as pipeline steps (a
 // step of the routed gate/up GEMM on single CTAs, 0.42 us, is the unit; the other rates are measured in that unit) times rounds.
-// us of the two GEMMs of the routed experts (gate/up + down), single CTAs / pairs: 2048 x 11008, 16 experts, top-2: 134 / 172 (768
-// tokens), 180 / 176 (960), 285 / 248 (2048); 4 experts, top-1: 96 / 80 (768); 896 x 4864, 4 experts: 54 / 60 (1024), 92 / 92 (2304),
-// 126 / 117 (4096); 512 x 2048, 16 experts: 62 / 68 (4096).  Of the shared ones: 2048 x 11008: 127 / 143 (1152: K splits fill one
-// round of single CTAs), 182 / 166 (1536); 256 x 512: 39 / 43 (8192).
+// us of the two GEMMs of the routed experts (gate/up + down), single CTAs / pairs, uniform routing: 2048 x 11008, 16 experts, top-2:
+// 131 / 178 (768 tokens), 132 / 182 (960), 230 / 183 (1536), 290 / 256 (2048); 4 experts, top-1: 88 / 74 (768), 102 / 102 (1152);
+// 896 x 4864, 4 experts: 48 / 48 (1024), 86 / 84 (2304), 122 / 109 (4096); 512 x 2048, 16 experts: 54 / 59 (4096); 384 x 9216,
+// 2 experts, top-1: 94 / 85 (4000).  Of the shared ones: 2048 x 11008: 125 / 142 (1152: K splits fill one round of single CTAs),
+// 174 / 163 (1536); 256 x 512: 33 / 35 (8192).
+// The rule errs towards single CTAs where an expert's rows lie below 256, of which half a tile per expert is too much (it forgoes
+// the pairs at 16 experts, 1536 tokens, and at 4 experts, 768 tokens), and once the other way (256 x 512, 8192 tokens: 32 / 34).
+// It puts a routed down projection at pick_bn's width, although few row tiles are launched narrower (setup_ternary), and the
+// two GEMMs of a step share a table of tiles, so they choose alike.
 // ------------------------------------------------------------------------------------------------
 static double gemm_steps(double row_tiles, int n_tiles, double steps, int workers, bool halves, double per_step, double least) {
   const double rounds = row_tiles * n_tiles / workers, whole = std::floor(rounds + 1e-9), tail = rounds - whole;
